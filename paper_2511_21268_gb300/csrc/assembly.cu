@@ -30,17 +30,20 @@
 // kappa = exp(g), g = sigma sqrt(2/M) sum_m cos(omega_m . x + phi_m) with
 // x = (x(xi1, xi2), y(xi1, xi2), z(xi3)): cos(a + b) = cos a cos b - sin a sin b
 // separates the plane and z parts, so g at all Q^3 points is the product of
-// a Q^2 x 2M matrix [cos a, -sin a] and a 2M x Q matrix [cos b; sin b] -- an
-// FP64 GEMM (register-tiled, below) whose epilogue forms the coefficients.
+// a Q^2 x 2M matrix [cos a, -sin a] and a 2M x Q matrix [cos b; sin b].  Its
+// entries lie in [-1, 1], so it runs exactly enough in fixed point on the
+// FP16 tensor cores (k_iga_coef_gemm below).
 //
-// Everything is FP64.  The sums run in a different order than an element
+// Everything else is FP64.  The sums run in a different order than an element
 // loop's, so results agree with one to rounding, not bit for bit.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
 #include <cmath>
+#include <numeric>
 #include <type_traits>
 #include <vector>
 
@@ -57,7 +60,13 @@ constexpr int kCtIn = 32;        // inner positions per block of the contraction
 constexpr int kCtWarps = 8;      // warps per block of the contractions
 constexpr int kInRows = 8;       // rows per block of the last contraction
 constexpr int kGT = 64;          // GEMM tile (plane points x z points)
-constexpr int kGK = 16;          // GEMM depth per stage
+constexpr int kGK = 32;          // GEMM depth per stage
+constexpr int kGStages = 3;      // stages in the copy ring
+constexpr int kSlices = 8;       // fixed-point digits per GEMM operand
+constexpr int kDigitBits = 7;
+constexpr int kFixBits = 55;     // operands are rounded to multiples of 2^-55
+constexpr int64_t kDigitBytes = 96LL << 20;  // digits of one piece of the plane
+constexpr int kFlushK = 256;     // products between two flushes of the FP32 accumulators
 
 struct IgaDims {
     int n, p, nq, m, off, Q, B, R, Lmax, R1, L1max;
@@ -195,9 +204,11 @@ __global__ void k_iga_single(IgaDims d, const double* __restrict__ V, int* s, in
 }
 
 // Plane data per point (q2, q1) of the (xi1, xi2) plane, p2 = q2 Q + q1:
-// x, y, the 2x2 block G = J2^-1 J2^-T (g00, g01, g11) and |det J2| w1 w2 (h/2)^2.
+// x, y, the 2x2 block G = J2^-1 J2^-T (g00, g01, g11), |det J2| w1 w2 (h/2)^2
+// and 3 pi^2 sin(pi x) sin(pi y).
 // geometry 0: identity; 1: quarter annulus, (1 + xi1) c(xi2) with c the
 // quadratic NURBS arc through (1,0), (1,1), (0,1), weights 1, sqrt(1/2), 1.
+constexpr int kPlane = 7;
 __global__ void k_iga_plane(int geometry, int n, int nq, const double* __restrict__ gx,
                             const double* __restrict__ gw, double* plane) {
     const int Q = n * nq;
@@ -236,55 +247,103 @@ __global__ void k_iga_plane(int geometry, int n, int nq, const double* __restric
     const double det = j00 * j11 - j01 * j10;
     // J2^-1 = [j11 -j01; -j10 j00] / det; G = J2^-1 J2^-T (rows of J2^-1 dotted)
     const double a = j11 / det, b = -j01 / det, c = -j10 / det, dd = j00 / det;
-    double* o = plane + p2 * 6;
+    double* o = plane + p2 * kPlane;
     o[0] = x;
     o[1] = y;
     o[2] = a * a + b * b;
     o[3] = a * c + b * dd;
     o[4] = c * c + dd * dd;
     o[5] = fabs(det) * w;
+    const double pi = 3.14159265358979323846;
+    o[6] = 3.0 * pi * pi * sin(pi * x) * sin(pi * y);  // the sine source's plane factor
 }
 
-// z and w3 (h/2) per z point.
+// z, w3 (h/2) and sin(pi z) per z point.
+constexpr int kZline = 3;
 __global__ void k_iga_zline(int n, int nq, const double* __restrict__ gx, const double* __restrict__ gw,
                             double* zl) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n * nq) return;
     const double h = 1.0 / n;
-    zl[2 * q] = (q / nq + 0.5 * (gx[q % nq] + 1.0)) * h;
-    zl[2 * q + 1] = 0.5 * h * gw[q % nq];
+    const double z = (q / nq + 0.5 * (gx[q % nq] + 1.0)) * h;
+    zl[kZline * q] = z;
+    zl[kZline * q + 1] = 0.5 * h * gw[q % nq];
+    zl[kZline * q + 2] = sin(3.14159265358979323846 * z);
 }
 
-// GEMM operands of kappa: Ak[p2][k] = cos(a_m) (k = m < M), -sin(a_m)
-// (k = M + m), zero padding up to K2; Bk[k][q3] = cos(b_m), sin(b_m).
-// a_m = omega_m,x x + omega_m,y y + phi_m, b_m = omega_m,z z.
-__global__ void k_iga_kappa_plane(int64_t P2, int M, int K2, const double* __restrict__ plane,
-                                  const double* __restrict__ om, const double* __restrict__ ph, double* Ak) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= P2 * K2) return;
-    const int64_t p2 = idx / K2;
-    const int k = (int)(idx % K2);
-    double v = 0.0;
-    if (k < 2 * M) {
-        const int mm = k % M;
-        const double a = om[3 * mm] * plane[p2 * 6] + om[3 * mm + 1] * plane[p2 * 6 + 1] + ph[mm];
-        v = k < M ? cos(a) : -sin(a);
+// ------------------------------------------------ kappa on the tensor cores
+// g = sum_k A[p2][k] B[q3][k] over K2 columns: k < M the cosines, M <= k < 2 M
+// the (negated) sines, the rest zero.  GB300 adds about two FP64 products per
+// SM and clock (16.3 ms for the 8.6 G products of n = 64, p = 3, M = 256, the
+// largest part of the assembly), its FP16 tensor cores about a thousand, so
+// the product runs in fixed point: every operand is rounded to a multiple of
+// 2^-55 (|x| <= 1, so closer than cos and sin themselves are) and split into
+// eight balanced base-128 digits, |digit| <= 64, each exact in FP16.  Digit
+// products are integers of at most 2^12; the FP32 accumulators of the tensor
+// cores add them exactly as long as the sums stay below 2^24, so the products
+// of all digit pairs (i, j) with the same weight i + j = t share accumulator t
+// and are flushed every kFlushK columns (8 pairs x 256 x 2^12 = 2^23) into a
+// 64-bit integer.  Pairs with i + j > 7 are left out: they weigh at most
+// 2^-56, and over all columns add about sqrt(7 K2) 2^-58.  What remains is
+// the operands' rounding, about sqrt(2 K2) 2^-57: below the rounding of an
+// FP64 sum of K2 such terms, whose partial sums reach sqrt(K2 / 2).
+// (Splitting FP64 products into exact low-precision products: Ootomo, Ozaki
+// and Yokota, "DGEMM on integer matrix multiplication unit", 2024, and
+// Mukunoki et al., "DGEMM using tensor cores", 2020.)
+
+// The digits of x, most significant first, stored kSlices arrays of `stride`
+// apart; a value that is not finite becomes a NaN in the first digit.
+__device__ __forceinline__ void store_digits(double x, __half* out, int64_t stride) {
+    long long X = __double2ll_rn(x * (double)(1LL << kFixBits));
+    __half d[kSlices];
+    constexpr int kHalf = 1 << (kDigitBits - 1), kMask = (1 << kDigitBits) - 1;
+#pragma unroll
+    for (int t = kSlices - 1; t > 0; t--) {
+        const int v = ((int)(X + kHalf) & kMask) - kHalf;
+        d[t] = __int2half_rn(v);
+        X = (X - v) >> kDigitBits;
     }
-    Ak[idx] = v;
+    d[0] = isfinite(x) ? __int2half_rn((int)X) : __ushort_as_half(0x7fff);
+#pragma unroll
+    for (int t = 0; t < kSlices; t++) out[t * stride] = d[t];
 }
 
+// Digits of A for the plane points [p0, p0 + rows): column m < M holds
+// cos(a_m), column M + m holds -sin(a_m), a_m = omega_m,x x + omega_m,y y +
+// phi_m.  Thread per (point, m), m padded to K2 - M (the padding is zero).
+__global__ void k_iga_kappa_plane(int64_t p0, int rows, int M, int K2, const double* __restrict__ plane,
+                                  const double* __restrict__ om, const double* __restrict__ ph, __half* As) {
+    const int W = K2 - M;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (int64_t)rows * W) return;
+    const int row = (int)(idx / W), mm = (int)(idx % W);
+    const int64_t stride = (int64_t)rows * K2;
+    __half* o = As + (int64_t)row * K2;
+    if (mm < M) {
+        const double* pl = plane + (p0 + row) * kPlane;
+        const double a = om[3 * mm] * pl[0] + om[3 * mm + 1] * pl[1] + ph[mm];
+        double sn, cs;
+        sincos(a, &sn, &cs);
+        store_digits(cs, o + mm, stride);
+        store_digits(-sn, o + M + mm, stride);
+    } else {
+        store_digits(0.0, o + M + mm, stride);
+    }
+}
+
+// Digits of B, [q3][k]: cos(b_m), sin(b_m), b_m = omega_m,z z.
 __global__ void k_iga_kappa_z(int Q, int M, int K2, const double* __restrict__ zl, const double* __restrict__ om,
-                              double* Bk) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= K2 * Q) return;
-    const int k = idx / Q, q3 = idx % Q;
+                              __half* Bs) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (int64_t)K2 * Q) return;
+    const int q3 = (int)(idx / K2), k = (int)(idx % K2);
     double v = 0.0;
     if (k < 2 * M) {
         const int mm = k % M;
-        const double b = om[3 * mm + 2] * zl[2 * q3];
+        const double b = om[3 * mm + 2] * zl[kZline * q3];
         v = k < M ? cos(b) : sin(b);
     }
-    Bk[idx] = v;
+    store_digits(v, Bs + idx, (int64_t)K2 * Q);
 }
 
 struct CoefOut {
@@ -295,22 +354,15 @@ struct CoefOut {
 __device__ __forceinline__ void coef_store(const CoefOut& o, int64_t P2, int64_t p2, int q3, double g, double amp,
                                            const double* __restrict__ plane, const double* __restrict__ zl,
                                            int source) {
-    const double* pl = plane + p2 * 6;
-    const double dw = pl[5] * zl[2 * q3 + 1];
+    const double* pl = plane + p2 * kPlane;
+    const double dw = pl[5] * zl[kZline * q3 + 1];
     const double cw = (amp != 0.0 ? exp(amp * g) : 1.0) * dw;
     const int64_t at = (int64_t)q3 * P2 + p2;
     o.c00[at] = cw * pl[2];
     if (o.c01) o.c01[at] = cw * pl[3];
     o.c11[at] = cw * pl[4];
     o.c22[at] = cw;
-    if (o.e) {
-        double f = 1.0;
-        if (source == AMG_SRC_SINE) {
-            const double pi = 3.14159265358979323846;
-            f = 3.0 * pi * pi * sin(pi * pl[0]) * sin(pi * pl[1]) * sin(pi * zl[2 * q3]);
-        }
-        o.e[at] = f * dw;
-    }
+    if (o.e) o.e[at] = (source == AMG_SRC_SINE ? pl[6] * zl[kZline * q3 + 2] : 1.0) * dw;
 }
 
 // Coefficients without kappa (thread per point).
@@ -321,52 +373,140 @@ __global__ void k_iga_coef_const(int64_t P2, int Q, const double* __restrict__ p
     coef_store(o, P2, idx % P2, (int)(idx / P2), 0.0, 0.0, plane, zl, source);
 }
 
-// g[q3][p2] = sum_k Ak[p2][k] Bk[k][q3] on 64 x 64 tiles (256 threads, 4 x 4
-// accumulators each: rows tx + 16 a, columns ty + 16 b), then the
-// coefficients.  K2 is a multiple of kGK.
-__global__ void __launch_bounds__(256) k_iga_coef_gemm(int64_t P2, int Q, int K2, const double* __restrict__ Ak,
-                                                      const double* __restrict__ Bk, double amp,
-                                                      const double* __restrict__ plane,
-                                                      const double* __restrict__ zl, int source, CoefOut o) {
-    __shared__ double As[kGK][kGT + 1];
-    __shared__ double Bs[kGK][kGT];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t r0 = (int64_t)blockIdx.x * kGT;
-    const int c0 = blockIdx.y * kGT;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < K2; k0 += kGK) {
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// One stage: the kSlices digits of 64 A rows and 64 B rows, 32 columns (64
+// bytes) each.  A row's four 16-byte pieces are stored at piece ^ ((row >> 1)
+// & 3), so that the eight rows of an ldmatrix fall into different banks.
+constexpr int kGRowBytes = kGK * 2;
+constexpr int kGOperand = kSlices * kGT * kGRowBytes;
+constexpr int kGStageBytes = 2 * kGOperand;
+__device__ __forceinline__ int tile_at(int slice, int row, int piece) {
+    return (slice * kGT + row) * kGRowBytes + ((piece ^ ((row >> 1) & 3)) << 4);
+}
+
+// g on 64 x 64 tiles (plane points p0 + r0 .., z points c0 ..), then the
+// coefficients.  8 warps of 32 x 16 outputs: per 16 columns a warp loads the
+// eight digits of its 16 B columns (32 registers) and, one at a time, of its
+// 32 A rows, and issues 36 digit pairs x 4 MMAs.  Blocks of the same plane
+// points run next to each other (x: the z tiles), so A's digits come from L2.
+// Measured at n = 64, p = 3, M = 256: digits 1.06 ms (bound by cos and sin in
+// FP64), product with the coefficients 2.24 ms (36 digit products, 0.31 P
+// multiply-adds; the coefficients' exp and FP64 products are about half of
+// it), against 1.39 and 16.34 ms in FP64.  The whole assembly 30.0 -> 16.6 ms,
+// with the error against a dense FP64 contraction 7.4e-16 before and 7.3e-16
+// after.
+__global__ void __launch_bounds__(256, 1) k_iga_coef_gemm(int64_t P2, int64_t p0, int rows, int Q, int K2, int fix,
+                                                         const __half* __restrict__ As,
+                                                         const __half* __restrict__ Bs, double amp,
+                                                         const double* __restrict__ plane,
+                                                         const double* __restrict__ zl, int source, CoefOut o) {
+    extern __shared__ __align__(128) unsigned char stage[];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int r0 = blockIdx.y * kGT, c0 = blockIdx.x * kGT;
+    const uint32_t base = smem_addr(stage);
+    const int64_t astride = (int64_t)rows * K2, bstride = (int64_t)Q * K2;
+    // rows past the operands' ends repeat the last one (their outputs are not stored)
+    auto load = [&](int buf, int k0) {
+        const uint32_t dst = base + buf * kGStageBytes;
 #pragma unroll
-        for (int u = 0; u < (kGT * kGK) / 256; u++) {
-            const int e = tid + 256 * u;
-            const int row = e / kGK, kk = e % kGK;
-            As[kk][row] = r0 + row < P2 ? Ak[(r0 + row) * K2 + k0 + kk] : 0.0;
-            const int kb = e / kGT, col = e % kGT;
-            Bs[kb][col] = c0 + col < Q ? Bk[(int64_t)(k0 + kb) * Q + c0 + col] : 0.0;
+        for (int u = 0; u < kSlices * kGT * 4 / 256; u++) {
+            const int e = tid + 256 * u, piece = e & 3, row = (e >> 2) & (kGT - 1), sl = e / (4 * kGT);
+            const int ra = min(r0 + row, rows - 1), rb = min(c0 + row, Q - 1);
+            const int at = tile_at(sl, row, piece);
+            copy16(dst + at, As + sl * astride + (int64_t)ra * K2 + k0 + piece * 8);
+            copy16(dst + kGOperand + at, Bs + sl * bstride + (int64_t)rb * K2 + k0 + piece * 8);
         }
-        __syncthreads();
+    };
+    const int wm = (wid & 1) * 32, wn = (wid >> 1) * 16;
+    float acc[kSlices][2][2][4];
+    long long tot[2][2][4];
+    unsigned bad = 0;
 #pragma unroll
-        for (int kk = 0; kk < kGK; kk++) {
-            double a[4], b[4];
+    for (int t = 0; t < kSlices; t++)
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                a[u] = As[kk][tx + 16 * u];
-                b[u] = Bs[kk][ty + 16 * u];
-            }
+        for (int i = 0; i < 16; i++) acc[t][i >> 3][(i >> 2) & 1][i & 3] = 0.f;
 #pragma unroll
-            for (int u = 0; u < 4; u++)
+    for (int i = 0; i < 16; i++) tot[i >> 3][(i >> 2) & 1][i & 3] = 0;
+    const int nk = K2 / kGK;
 #pragma unroll
-                for (int v = 0; v < 4; v++) acc[u][v] = fma(a[u], b[v], acc[u][v]);
-        }
-        __syncthreads();
+    for (int b = 0; b < kGStages - 1; b++) {
+        if (b < nk) load(b, b * kGK);
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
+    for (int kt = 0; kt < nk; kt++) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kGStages - 2) : "memory");
+        __syncthreads();
+        if (kt + kGStages - 1 < nk) load((kt + kGStages - 1) % kGStages, (kt + kGStages - 1) * kGK);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const uint32_t src = base + (kt % kGStages) * kGStageBytes;
 #pragma unroll
-    for (int u = 0; u < 4; u++)
+        for (int ks = 0; ks < kGK / 16; ks++) {
+            uint32_t b[kSlices][4];
 #pragma unroll
-        for (int v = 0; v < 4; v++) {
-            const int64_t p2 = r0 + tx + 16 * u;
-            const int q3 = c0 + ty + 16 * v;
-            if (p2 < P2 && q3 < Q) coef_store(o, P2, p2, q3, acc[u][v], amp, plane, zl, source);
+            for (int j = 0; j < kSlices; j++)
+                ldmatrix4(b[j], src + kGOperand + tile_at(j, wn + (lane & 7) + ((lane >> 4) << 3),
+                                                          ks * 2 + ((lane >> 3) & 1)));
+#pragma unroll
+            for (int i = 0; i < kSlices; i++) {
+                uint32_t a[2][4];
+#pragma unroll
+                for (int mi = 0; mi < 2; mi++)
+                    ldmatrix4(a[mi], src + tile_at(i, wm + mi * 16 + (lane & 15), ks * 2 + (lane >> 4)));
+#pragma unroll
+                for (int j = 0; j < kSlices - i; j++)
+#pragma unroll
+                    for (int mi = 0; mi < 2; mi++) {
+                        mma_f16(acc[i + j][mi][0], a[mi], b[j][0], b[j][1]);
+                        mma_f16(acc[i + j][mi][1], a[mi], b[j][2], b[j][3]);
+                    }
+            }
         }
+        if ((kt + 1) % (kFlushK / kGK) == 0 || kt + 1 == nk) {
+            // weight of accumulator t: 2^(2 x 49 - 7 t - 2 x 55) = 2^-(12 + 7 t),
+            // in units of 2^-fix
+#pragma unroll
+            for (int i = 0; i < 16; i++) {
+                const int mi = i >> 3, ni = (i >> 2) & 1, e = i & 3;
+                if (isnan(acc[0][mi][ni][e])) bad |= 1u << i;
+                long long s = 0;
+#pragma unroll
+                for (int t = 0; t < kSlices; t++) {
+                    const long long v = (long long)__float2int_rn(acc[t][mi][ni][e]);
+                    const int sh = fix - 2 * (kFixBits - kDigitBits * (kSlices - 1)) - kDigitBits * t;
+                    s += sh >= 0 ? v << sh : (v + (1LL << (-sh - 1))) >> -sh;
+                    acc[t][mi][ni][e] = 0.f;
+                }
+                tot[mi][ni][e] += s;
+            }
+        }
+    }
+    const double unit = __longlong_as_double((long long)(1023 - fix) << 52);
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        const int mi = i >> 3, ni = (i >> 2) & 1, e = i & 3;
+        const int row = r0 + wm + mi * 16 + (lane >> 2) + (e >> 1) * 8;
+        const int q3 = c0 + wn + ni * 8 + (lane & 3) * 2 + (e & 1);
+        if (row < rows && q3 < Q) {
+            const double g = bad >> i & 1u ? __longlong_as_double(0x7ff8000000000000LL) : (double)tot[mi][ni][e] * unit;
+            coef_store(o, P2, p0 + row, q3, g, amp, plane, zl, source);
+        }
+    }
 }
 
 // Contraction of the middle (outer-major) axis: Y[o][r][c] (+)= sum_{k < L[r]}
@@ -623,8 +763,8 @@ extern "C" int amg_iga_assemble(const amg_iga_patch* P, int64_t* rowptr, int32_t
     get(&gw, d.nq);
     get(&V, (size_t)Q * (d.p + 1));
     get(&D, (size_t)Q * (d.p + 1));
-    get(&plane, (size_t)P2 * 6);
-    get(&zl, (size_t)Q * 2);
+    get(&plane, (size_t)P2 * kPlane);
+    get(&zl, (size_t)Q * kZline);
     for (auto& w : Wt) get(&w, (size_t)R * d.Lmax);
     get(&W1, (size_t)d.R1 * d.L1max);
     get(&sp, R);
@@ -650,19 +790,43 @@ extern "C" int amg_iga_assemble(const amg_iga_patch* P, int64_t* rowptr, int32_t
     if (err != cudaSuccess) return report_cuda(err, "amg_iga_assemble coefficients");
     double gemm_fma = 0.0;
     if (M > 0) {
-        double *Ak, *Bk;
-        get(&Ak, (size_t)P2 * K2);
-        get(&Bk, (size_t)K2 * Q);
+        // A's digits in pieces of about kDigitBytes (64 rows at least), so that
+        // they stay in L2 between the kernel that writes them and the product
+        __half *As, *Bs;
+        const int64_t row_bytes = (int64_t)kSlices * K2 * sizeof(__half);
+        int64_t tiles = std::min<int64_t>((P2 + kGT - 1) / kGT, std::max<int64_t>(1, kDigitBytes / (row_bytes * kGT)));
+        const int ct = (Q + kGT - 1) / kGT;
+        int dev = 0, sms = 1;
+        if ((err = cudaGetDevice(&dev)) != cudaSuccess ||
+            (err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+            return report_cuda(err, "amg_iga_assemble device");
+        // whole waves of blocks (one per SM) where a piece has at least one
+        const int64_t wave = sms / std::gcd(sms, ct);
+        if (tiles >= wave && tiles * kGT < P2) tiles -= tiles % wave;
+        const int64_t chunk = tiles * kGT;
+        get(&As, (size_t)(std::min(chunk, P2) * row_bytes / sizeof(__half)));
+        get(&Bs, (size_t)kSlices * K2 * Q);
         if (err != cudaSuccess) return report_cuda(err, "amg_iga_assemble kappa");
-        k_iga_kappa_plane<<<AMG_GRID(nblk(P2 * K2, 256)), 256, 0, s>>>(P2, M, K2, plane, P->kappa_omega,
-                                                                          P->kappa_phi, Ak);
-        k_iga_kappa_z<<<AMG_GRID(nblk((int64_t)K2 * Q, 256)), 256, 0, s>>>(Q, M, K2, zl, P->kappa_omega, Bk);
+        const size_t smg = (size_t)kGStages * kGStageBytes;
+        if ((err = cudaFuncSetAttribute(k_iga_coef_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smg)) !=
+            cudaSuccess)
+            return report_cuda(err, "amg_iga_assemble smem");
+        k_iga_kappa_z<<<AMG_GRID(nblk((int64_t)K2 * Q, 256)), 256, 0, s>>>(Q, M, K2, zl, P->kappa_omega, Bs);
         const double amp = P->kappa_sigma * sqrt(2.0 / M);
-        dim3 grid((unsigned)((P2 + kGT - 1) / kGT), (unsigned)((Q + kGT - 1) / kGT));
-        k_iga_coef_gemm<<<AMG_GRID(grid), 256, 0, s>>>(P2, Q, K2, Ak, Bk, amp, plane, zl, P->source, co);
+        // |g| <= 2 M < 2^(62 - fix): the 64-bit sums cannot overflow
+        int fix = 53;
+        while (fix > 32 && (1LL << (62 - fix)) <= 2 * (int64_t)M) fix--;
+        for (int64_t p0 = 0; p0 < P2; p0 += chunk) {
+            const int rows = (int)std::min(chunk, P2 - p0);
+            k_iga_kappa_plane<<<AMG_GRID(nblk((int64_t)rows * (K2 - M), 256)), 256, 0, s>>>(
+                p0, rows, M, K2, plane, P->kappa_omega, P->kappa_phi, As);
+            dim3 grid((unsigned)((Q + kGT - 1) / kGT), (unsigned)((rows + kGT - 1) / kGT));
+            k_iga_coef_gemm<<<AMG_GRID(grid), 256, smg, s>>>(P2, p0, rows, Q, K2, fix, As, Bs, amp, plane, zl,
+                                                             P->source, co);
+        }
         gemm_fma = (double)P2 * Q * (2.0 * M);
-        release(Ak);
-        release(Bk);
+        release(As);
+        release(Bs);
     } else {
         k_iga_coef_const<<<AMG_GRID(nblk(P3, 256)), 256, 0, s>>>(P2, Q, plane, zl, P->source, co);
     }
