@@ -302,11 +302,13 @@ cudaError_t launch_to_bf16(const double* in, __nv_bfloat16* out, int64_t n, cuda
 // solve_kernels.cu
 cudaError_t launch_spmv(const DevCSR& A, const double* x, double* y, cudaStream_t s);
 cudaError_t enqueue_vcycle(amg_hierarchy* h, cudaStream_t s);
+// the same V-cycle with every matrix pass on the row-group kernels
+cudaError_t enqueue_vcycle_rows(amg_hierarchy* h, cudaStream_t s);
 cudaError_t enqueue_vcycle_standalone(amg_hierarchy* h, cudaStream_t s);
 cudaError_t enqueue_pcg_start(amg_hierarchy* h, cudaStream_t s);
 cudaError_t enqueue_pcg_iteration(amg_hierarchy* h, cudaStream_t s);
 cudaError_t launch_final_residual(amg_hierarchy* h, cudaStream_t s);
-cudaError_t launch_rowgroup_pq(amg_hierarchy* h, cudaStream_t s);
+cudaError_t launch_rowgroup_pq(amg_hierarchy* h, cudaStream_t s, bool batch = false);
 double* final_residual_slot(amg_hierarchy* h);
 // multi_solve.cu
 cudaError_t enqueue_multi_start(amg_hierarchy* h, cudaStream_t s);
@@ -385,6 +387,7 @@ cudaError_t launch_run_rows(const DevCSR& A, int32_t* runcnt, uint8_t* runlen, i
 cudaError_t launch_run_fill(const DevCSR& A, const int32_t* run_ptr, const uint8_t* runlen, int32_t* run_start,
                             cudaStream_t s);
 int rows_per_warp(int n, int num_sms);
+int level_rows(const amg_hierarchy* h, const Level& L, bool batch);
 int row_blocks(int n, int rpw);
 int vec_blocks(int n, int num_sms);
 size_t partial_slot_size(int n0, int num_sms);  // >= num_sms + 2

@@ -23,26 +23,26 @@ __device__ __forceinline__ double ldv(const double* v, int64_t k) { return __ldg
 __device__ __forceinline__ float ldv(const float* v, int64_t k) { return __ldg(v + k); }
 __device__ __forceinline__ float ldv(const __nv_bfloat16* v, int64_t k) { return __bfloat162float(v[k]); }
 
-// Lane partial of row i: sum over k = b + lane + 32 t of v_k x_{c_k}, in A.
-// The rows this runs on (levels with few rows, a warp per row) are
-// latency-bound: each chunk of U entries per lane loads all its values and
-// columns, then all its x entries, then runs the FMA chain in entry order,
-// and the last partial chunk does the same with predicated loads, so a row
-// of up to 32 U entries costs two dependent round trips.
-template <typename A, typename V, typename X>
+// Lane partial of row i: sum over k = b + lane + S t of v_k x_{c_k}, in A (S
+// lanes per row).  The rows this runs on (levels with few rows, short rows)
+// are latency-bound: each chunk of U entries per lane loads all its values
+// and columns, then all its x entries, then runs the FMA chain in entry
+// order, and the last partial chunk does the same with predicated loads, so a
+// row of up to S U entries costs two dependent round trips.
+template <int S, typename A, typename V, typename X>
 __device__ __forceinline__ A lane_partial(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                           const V* __restrict__ v, const X* __restrict__ x, int i, int lane) {
     constexpr int U = sizeof(A) == 4 ? 16 : 8;
     const int64_t b = rp[i], e = rp[i + 1];
     A acc = A(0);
     int64_t k = b + lane;
-    for (; k + 32 * (U - 1) < e; k += 32 * U) {
+    for (; k + S * (U - 1) < e; k += S * U) {
         A vv[U], xx[U];
         int cc[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
-            vv[u] = (A)ldv(v, k + 32 * u);
-            cc[u] = __ldg(ci + k + 32 * u);
+            vv[u] = (A)ldv(v, k + S * u);
+            cc[u] = __ldg(ci + k + S * u);
         }
 #pragma unroll
         for (int u = 0; u < U; u++) xx[u] = (A)x[cc[u]];
@@ -54,9 +54,9 @@ __device__ __forceinline__ A lane_partial(const int64_t* __restrict__ rp, const 
         int cc[U - 1];
 #pragma unroll
         for (int u = 0; u < U - 1; u++) {
-            const bool in = k + 32 * u < e;
-            vv[u] = in ? (A)ldv(v, k + 32 * u) : A(0);
-            cc[u] = in ? __ldg(ci + k + 32 * u) : -1;
+            const bool in = k + S * u < e;
+            vv[u] = in ? (A)ldv(v, k + S * u) : A(0);
+            cc[u] = in ? __ldg(ci + k + S * u) : -1;
         }
 #pragma unroll
         for (int u = 0; u < U - 1; u++) xx[u] = cc[u] >= 0 ? (A)x[cc[u]] : A(0);
@@ -66,6 +66,21 @@ __device__ __forceinline__ A lane_partial(const int64_t* __restrict__ rp, const 
     }
     return acc;
 }
+
+// A warp's scratch in the row-group kernels with RPW rows per warp.
+template <typename A, int RPW>
+struct RowTile {};
+template <typename A>
+struct RowTile<A, 8> {
+    A t[8][33];  // lane partials of each row
+};
+constexpr int kFoldBytes = 64;  // of one row's values per staged chunk
+template <typename A>
+struct RowTile<A, 32> {
+    static constexpr int kC = kFoldBytes / sizeof(A);  // entries of each row per chunk
+    A v[32][kC + 1];
+    int c[32][kC + 1];
+};
 
 // Matrix views of the row-group kernels.  CsrM: plain CSR.  RunM: CSR
 // values with run-encoded columns (every row a sequence of equal runs of L
@@ -87,7 +102,60 @@ struct CsrM {
     const V* __restrict__ v;
     template <typename A, typename X>
     __device__ __forceinline__ A partial(const X* __restrict__ x, int i, int lane) const {
-        return lane_partial<A>(rp, ci, v, x, i, lane);
+        return lane_partial<32, A>(rp, ci, v, x, i, lane);
+    }
+    // one of 8 lanes of row i
+    template <typename A, typename X>
+    __device__ __forceinline__ A sub(const X* __restrict__ x, int i, int q) const {
+        return lane_partial<8, A>(rp, ci, v, x, i, q);
+    }
+    // Row row0 + lane as one chain of products in entry order, a lane per row
+    // (0 past the last row).  The warp stages kC entries of each of its 32 rows
+    // at a time in shared memory, 32 / kC rows per load instruction, with the
+    // next chunk's entries in registers meanwhile; neighbouring rows of a
+    // tensor-product matrix read neighbouring vector entries, so the gathers
+    // of the 32 lanes coalesce.
+    template <typename A, typename X>
+    __device__ __forceinline__ A ordered(const X* __restrict__ x, int row0, int n, int lane,
+                                         RowTile<A, 32>& T) const {
+        constexpr int C = RowTile<A, 32>::kC, RI = 32 / C, NI = 32 / RI;  // rows per instruction, instructions
+        const int64_t b = row0 + lane < n ? rp[row0 + lane] : 0;
+        const int len = row0 + lane < n ? (int)(rp[row0 + lane + 1] - b) : 0;
+        const int longest = __reduce_max_sync(FULL, len);
+        const int sub = lane / C, o = lane % C;  // this lane loads entry o of rows sub, sub + RI, ...
+        A nv[NI];
+        int nc[NI];
+        auto load = [&](int k0) {
+#pragma unroll
+            for (int j = 0; j < NI; j++) {
+                const int r = j * RI + sub;
+                const int64_t rb = __shfl_sync(FULL, b, r);
+                const bool in = k0 + o < __shfl_sync(FULL, len, r);
+                nv[j] = in ? (A)ldv(v, rb + k0 + o) : A(0);
+                nc[j] = in ? __ldg(ci + rb + k0 + o) : 0;
+            }
+        };
+        A acc = A(0);
+        load(0);
+        for (int k0 = 0; k0 < longest; k0 += C) {
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < NI; j++) {
+                T.v[j * RI + sub][o] = nv[j];
+                T.c[j * RI + sub][o] = nc[j];
+            }
+            __syncwarp();
+            if (k0 + C < longest) load(k0 + C);
+            const int cnt = min(C, len - k0);
+            A xx[C];
+#pragma unroll
+            for (int u = 0; u < C; u++)
+                if (u < cnt) xx[u] = (A)x[T.c[lane][u]];
+#pragma unroll
+            for (int u = 0; u < C; u++)
+                if (u < cnt) acc = fma(T.v[lane][u], xx[u], acc);
+        }
+        return acc;
     }
     // Lane partials of the RPW rows row0 .. row0+RPW-1 into tile[r][lane]:
     // the warp streams the rows' contiguous entries, lane t taking entries
@@ -154,6 +222,14 @@ struct RunM {
     const V* __restrict__ v;
     template <typename A, typename X>
     __device__ __forceinline__ A partial(const X* __restrict__ x, int i, int lane) const {
+        return strided<32, A>(x, i, lane);
+    }
+    template <typename A, typename X>
+    __device__ __forceinline__ A sub(const X* __restrict__ x, int i, int q) const {
+        return strided<8, A>(x, i, q);
+    }
+    template <int S, typename A, typename X>
+    __device__ __forceinline__ A strided(const X* __restrict__ x, int i, int lane) const {
         const int64_t b = __ldg(rp + i), e = __ldg(rp + i + 1);
         const uint32_t L = rlen[i];
         const uint32_t mg = kRunMagic[L];
@@ -166,16 +242,16 @@ struct RunM {
             const uint32_t q = __umulhi(w, mg);
             return __ldg(rs + q) + (int)(w - q * L);
         };
-        for (; u + 96 < len; u += 128) {
-            const A v0 = (A)ldv(vr, u), v1 = (A)ldv(vr, u + 32), v2 = (A)ldv(vr, u + 64), v3 = (A)ldv(vr, u + 96);
-            const int c0 = col(u), c1 = col(u + 32), c2 = col(u + 64), c3 = col(u + 96);
+        for (; u + 3 * S < len; u += 4 * S) {
+            const A v0 = (A)ldv(vr, u), v1 = (A)ldv(vr, u + S), v2 = (A)ldv(vr, u + 2 * S), v3 = (A)ldv(vr, u + 3 * S);
+            const int c0 = col(u), c1 = col(u + S), c2 = col(u + 2 * S), c3 = col(u + 3 * S);
             const A x0 = (A)x[c0], x1 = (A)x[c1], x2 = (A)x[c2], x3 = (A)x[c3];
             acc = fma(v0, x0, acc);
             acc = fma(v1, x1, acc);
             acc = fma(v2, x2, acc);
             acc = fma(v3, x3, acc);
         }
-        for (; u < len; u += 32) acc = fma((A)ldv(vr, u), (A)x[col(u)], acc);
+        for (; u < len; u += S) acc = fma((A)ldv(vr, u), (A)x[col(u)], acc);
         return acc;
     }
 };
@@ -184,14 +260,29 @@ struct RunM {
 // Returns the total of row `row0 + lane / (32/RPW)` on every lane.
 template <int RPW, typename A, typename M, typename X>
 __device__ __forceinline__ A group_rows(const M& mat, const X* __restrict__ x, int row0, int n, int lane,
-                                        A (*tile)[33]) {
+                                        RowTile<A, RPW>& T) {
     if constexpr (RPW == 1) {
         A s = row0 < n ? mat.template partial<A>(x, row0, lane) : A(0);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
         return s;
+    } else if constexpr (RPW == 4) {
+        // 8 lanes per row: short rows, and levels whose rows are too few for
+        // groups of 8.  FP64 instructions are what a row costs (a warp
+        // instruction holds a quarter of an SM's FP64 pipe for 64 cycles): a
+        // row of 49 entries takes (7 products + 3 adds) / 4 of them here
+        // against 2 + 5 with a warp per row.
+        const int i = row0 + (lane >> 3);
+        A s = i < n ? mat.template sub<A>(x, i, lane & 7) : A(0);
+        __syncwarp();
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+        return s;
+    } else if constexpr (RPW == 32) {
+        return mat.template ordered<A>(x, row0, n, lane, T);
     } else {
         constexpr int LPR = 32 / RPW;  // lanes per row in the finishing step
+        A(*tile)[33] = T.t;
         if constexpr (M::kFlat) {
             mat.template flat<RPW, A>(x, row0, n, lane, tile);
         } else {
@@ -214,9 +305,12 @@ __device__ __forceinline__ A group_rows(const M& mat, const X* __restrict__ x, i
 }
 
 // Deterministic sum of one value per lane over the block -> *out (thread 0).
+// STEP: only every STEP-th lane holds a value (a row's owner), the others
+// zero, so the adds among them are left out.
+template <int STEP = 1>
 __device__ __forceinline__ void block_partial(double tv, double* sh, double* out) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tv += __shfl_xor_sync(FULL, tv, o);
+    for (int o = 16; o >= STEP; o >>= 1) tv += __shfl_xor_sync(FULL, tv, o);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
     if (lane == 0) sh[wid] = tv;
@@ -235,7 +329,7 @@ __device__ __forceinline__ void block_partial(double tv, double* sh, double* out
 
 // Common prologue of the row-group kernels.
 #define ROWGROUP_PROLOGUE(A)                                           \
-    __shared__ A tiles[kWarpsPerBlock][RPW][33];                       \
+    __shared__ RowTile<A, RPW> tiles[kWarpsPerBlock];                   \
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;         \
     const int row0 = (blockIdx.x * kWarpsPerBlock + wid) * RPW;        \
     constexpr int LPR = 32 / RPW;                                      \
@@ -264,7 +358,7 @@ __global__ void __launch_bounds__(kBlock) k_residual0(int n, M mat, const double
     // grid-stride over row groups (a small grid: the gated launch of every
     // mixed-precision iteration returns at once unless a replacement is due)
     if (gate && (gate->done || !gate->replace_now)) return;
-    __shared__ double tiles[kWarpsPerBlock][RPW][33];
+    __shared__ RowTile<double, RPW> tiles[kWarpsPerBlock];
     __shared__ double sh[kWarpsPerBlock];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int LPR = 32 / RPW;
@@ -282,12 +376,12 @@ __global__ void __launch_bounds__(kBlock) k_residual0(int n, M mat, const double
             ff += fi * fi;
         }
     }
-    block_partial(rr, sh, part_rr + blockIdx.x);
-    if (part_ff) block_partial(ff, sh, part_ff + blockIdx.x);
+    block_partial<LPR>(rr, sh, part_rr + blockIdx.x);
+    if (part_ff) block_partial<LPR>(ff, sh, part_ff + blockIdx.x);
 }
 
 // Outer SpMV q = K p (values V, gathered vector PX, accumulation A; q FP64),
-// partials p.q and (flexible) p.r with the FP64 p.
+// partials p.q and (flexible) p.r with the FP64 p (part_pq null: none).
 template <int RPW, typename A, typename M, typename PX>
 __global__ void __launch_bounds__(kBlock) k_spmv_pq(int n, M mat, const PX* __restrict__ pg,
                                                      const double* __restrict__ p,
@@ -302,12 +396,15 @@ __global__ void __launch_bounds__(kBlock) k_spmv_pq(int n, M mat, const PX* __re
     if (owner) {
         const double qs = (double)s;
         q[myrow] = qs;
-        const double pi = p[myrow];
-        pq = pi * qs;
-        if (flexible) pr = pi * r[myrow];
+        if (part_pq) {
+            const double pi = p[myrow];
+            pq = pi * qs;
+            if (flexible) pr = pi * r[myrow];
+        }
     }
-    block_partial(pq, sh, part_pq + blockIdx.x);
-    if (flexible) block_partial(pr, sh, part_pr + blockIdx.x);
+    if (!part_pq) return;
+    block_partial<LPR>(pq, sh, part_pq + blockIdx.x);
+    if (flexible) block_partial<LPR>(pr, sh, part_pr + blockIdx.x);
 }
 
 // rbuf = f - K x (down-sweep residual of one level).
@@ -334,19 +431,33 @@ __global__ void __launch_bounds__(kBlock) k_sweep(int n, M mat, const FT* __rest
 
 // Up sweep of level l >= 1: y_a = x_a + (f_a - (K x)_a) / d_a, then
 // x_{l-1}[c] += p_c y_a for the members c of a (one member per lane of the
-// row's lane group).
+// row's lane group; with a row per lane, the members of the warp's 32 rows,
+// which are consecutive in midx, go over the lanes, each finding its row's y
+// through its aggregate).
 template <int RPW, typename A, typename M>
 __global__ void __launch_bounds__(kBlock) k_up(int n, M mat, const A* __restrict__ f, const A* __restrict__ x,
                                                 const A* __restrict__ invd,
                                                 const int32_t* __restrict__ mptr, const int32_t* __restrict__ midx,
-                                                const double* __restrict__ pvalf, A* xf, const SolveState* st) {
+                                                const int32_t* __restrict__ aggf, const double* __restrict__ pvalf,
+                                                A* xf, const SolveState* st) {
     pdl_entry();
     DONE_GUARD(st);
     ROWGROUP_PROLOGUE(A)
     const A s = group_rows<RPW, A>(mat, x, row0, n, lane, tiles[wid]);
-    // every lane of the row's group has the total; the aggregate's members
-    // (independent fine rows) are spread over those LPR lanes
-    if (myrow < n) {
+    if constexpr (RPW == 32) {
+        if (row0 >= n) return;
+        const A y = myrow < n ? fma(invd[myrow], f[myrow] - s, x[myrow]) : A(0);
+        const int m1 = mptr[min(row0 + 32, n)];
+#pragma unroll 4
+        for (int m0 = mptr[row0]; m0 < m1; m0 += 32) {
+            const bool in = m0 + lane < m1;
+            const int c = in ? midx[m0 + lane] : 0;
+            const A ya = __shfl_sync(FULL, y, in ? aggf[c] - row0 : 0);
+            if (in) xf[c] = fma((A)pvalf[c], ya, xf[c]);
+        }
+    } else if (myrow < n) {
+        // every lane of the row's group has the total; the aggregate's members
+        // (independent fine rows) are spread over those LPR lanes
         const A y = fma(invd[myrow], f[myrow] - s, x[myrow]);
         const int m1 = mptr[myrow + 1];
         for (int m = mptr[myrow] + lane % LPR; m < m1; m += LPR) {
@@ -357,7 +468,7 @@ __global__ void __launch_bounds__(kBlock) k_up(int n, M mat, const A* __restrict
 }
 
 // Up sweep of level 0: z = x + (r - K x) / d (z FP64); partials r.z and
-// (flexible) z.q.
+// (flexible) z.q (part_rz null: none).
 template <int RPW, typename A, typename M>
 __global__ void __launch_bounds__(kBlock) k_up0(int n, M mat, const double* __restrict__ r,
                                                  const A* __restrict__ x, const A* __restrict__ invd, double* z,
@@ -373,11 +484,14 @@ __global__ void __launch_bounds__(kBlock) k_up0(int n, M mat, const double* __re
         const double ra = r[myrow];
         const double za = (double)fma(invd[myrow], (A)ra - s, x[myrow]);
         z[myrow] = za;
-        rz = ra * za;
-        if (flexible) zq = za * q[myrow];
+        if (part_rz) {
+            rz = ra * za;
+            if (flexible) zq = za * q[myrow];
+        }
     }
-    block_partial(rz, sh, part_rz + blockIdx.x);
-    if (flexible) block_partial(zq, sh, part_zq + blockIdx.x);
+    if (!part_rz) return;
+    block_partial<LPR>(rz, sh, part_rz + blockIdx.x);
+    if (flexible) block_partial<LPR>(zq, sh, part_zq + blockIdx.x);
 }
 
 }  // namespace

@@ -506,8 +506,13 @@ __global__ void k_sqrt_sum(const double* part, int nb, double* out) {
 }
 
 // ----------------------------------------------------------------- dispatch
-template <typename F>
+// f(rows per warp) for matrix view M; 4 and 32 rows only on plain CSR
+template <typename M, typename F>
 inline void with_rpw(int rpw, F&& f) {
+    if constexpr (M::kFlat) {
+        if (rpw == 4) return f(std::integral_constant<int, 4>{});
+        if (rpw == 32) return f(std::integral_constant<int, 32>{});
+    }
     if (rpw == 8) f(std::integral_constant<int, 8>{});
     else f(std::integral_constant<int, 1>{});
 }
@@ -517,6 +522,29 @@ inline void with_rpw(int rpw, F&& f) {
 int rows_per_warp(int n, int num_sms) {
     // 8-row groups once there are enough of them to fill the GPU several times
     return ((int64_t)n >= (int64_t)num_sms * kWarpsPerBlock * 8 * 4) ? 8 : 1;
+}
+
+// Rows per warp of a level's row-group kernels in a single solve (batch = 0)
+// or a batch.  FP64 sums may be split over lanes in any way (the difference is
+// their rounding): short rows (at most kShortRow entries on average) take 8
+// lanes each, 4 rows per warp, where there is a warp's work for every SM, and
+// a lane each where there are kShortFull rows per SM.  Measured in FP64: 2-D
+// p = 3 n = 101 (49 entries), q = K p 14.2 -> 5.2 us and the level-0 up sweep
+// 15.2 -> 5.6 us with 4 rows per warp instead of one; the coarse levels of 3-D
+// p = 2 n = 49 (75 to 95 entries) 95 -> 75 us per V-cycle; no gain at 226
+// entries, a loss at 1,200 (a Chebyshev step 18 -> 29 us).  FP32 keeps the
+// split of rows_per_warp in a single solve.  A batch in FP32 sums every row in
+// entry order (a lane per row): mixed-precision solutions of ill-conditioned
+// systems show in the ninth digit how their V-cycle rounds.
+constexpr int kShortRow = 128;
+constexpr int kShortFull = 512;
+int level_rows(const amg_hierarchy* h, const Level& L, bool batch) {
+    const int64_t n = L.A.n, sms = h->num_sms;
+    const int plain = rows_per_warp(L.A.n, h->num_sms);
+    if (n == 0) return plain;
+    if (h->mixed) return batch ? 32 : plain;
+    if (L.A.nnz > kShortRow * n || n < sms * 4) return plain;
+    return n >= sms * kShortFull ? 32 : 4;
 }
 
 int row_blocks(int n, int rpw) {
@@ -543,7 +571,7 @@ cudaError_t launch_spmv(const DevCSR& A, const double* x, double* y, cudaStream_
     const int rpw = rows_per_warp(A.n, sms);
     const int nb = row_blocks(A.n, rpw);
     if (A.n == 0) return cudaSuccess;
-    with_rpw(rpw, [&](auto R) {
+    with_rpw<CsrM<double>>(rpw, [&](auto R) {
         launch_pdl(k_spmv<decltype(R)::value, CsrM<double>>, nb, kBlock, 0, s, A.n, CsrM<double>{A.rowptr, A.col, A.val}, x, y);
     });
     return cudaGetLastError();
@@ -562,10 +590,11 @@ enum { S_RR = 0, S_FF, S_PQ, S_PR, S_RZ, S_ZQ, S_OUT, S_RR2, S_COUNT };
 
 // ---------------------------------------------------------- per-mode views
 // Matrix view of level L with values v: run-encoded columns when the level
-// has them, plain CSR otherwise.
+// has them, plain CSR otherwise and for the kernels with 4 rows per warp
+// (short rows: decoding the runs costs more than reading the columns).
 template <typename V, typename Fn>
-static void with_mat(const Level& L, const V* v, Fn&& fn) {
-    if (L.run_ptr) fn(RunM<V>{L.A.rowptr, L.run_ptr, L.run_len, L.run_start, v});
+static void with_mat(const Level& L, const V* v, int rpw, Fn&& fn) {
+    if (L.run_ptr && rpw != 4 && rpw != 32) fn(RunM<V>{L.A.rowptr, L.run_ptr, L.run_len, L.run_start, v});
     else fn(CsrM<V>{L.A.rowptr, L.A.col, v});
 }
 
@@ -580,7 +609,7 @@ struct View<double> {
     static double* t(Level& L) { return L.t; }
     static const double* invd(Level& L) { return L.invd; }
     template <typename Fn>
-    static void vals(Level& L, int, Fn&& fn) { with_mat(L, static_cast<const double*>(L.A.val), fn); }
+    static void vals(Level& L, int, int rpw, Fn&& fn) { with_mat(L, static_cast<const double*>(L.A.val), rpw, fn); }
 };
 
 template <>
@@ -590,9 +619,9 @@ struct View<float> {
     static float* t(Level& L) { return L.t32; }
     static const float* invd(Level& L) { return L.invd32; }
     template <typename Fn>
-    static void vals(Level& L, int l, Fn&& fn) {
-        if (l == 0 && L.val16) with_mat(L, static_cast<const __nv_bfloat16*>(L.val16), fn);
-        else with_mat(L, static_cast<const float*>(L.val32), fn);
+    static void vals(Level& L, int l, int rpw, Fn&& fn) {
+        if (l == 0 && L.val16) with_mat(L, static_cast<const __nv_bfloat16*>(L.val16), rpw, fn);
+        else with_mat(L, static_cast<const float*>(L.val32), rpw, fn);
     }
 };
 
@@ -628,9 +657,11 @@ static void coarsest_solve(amg_hierarchy* h, A* xF, cudaStream_t s) {
 }
 
 // V-cycle on r (= f_0); the pre-smoothed level-0 iterate is already in x_0.
-// Writes z (FP64) and the partial sums of r.z (and z.q).
+// Writes z (FP64) and the partial sums of r.z (and z.q).  rows_only: every
+// matrix pass on the row-group kernels, also where the levels have sliced or
+// staged copies, and (on more than one level) no partial sums.
 template <typename A>
-static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s) {
+static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s, bool rows_only = false) {
     using Vw = View<A>;
     const int L = h->nlev;
     const int sms = h->num_sms;
@@ -653,15 +684,15 @@ static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s) {
         Level& F = h->lev[l];
         Level& C = h->lev[l + 1];
         const int n = F.A.n;
-        const int rpw = rows_per_warp(n, sms), nb = row_blocks(n, rpw);
-        Vw::vals(F, l, [&](auto mat) {
+        const int rpw = level_rows(h, F, rows_only), nb = row_blocks(n, rpw);
+        Vw::vals(F, l, rpw, [&](auto mat) {
             using M = decltype(mat);
             auto sweep_and_resid = [&](auto fp) {
                 using FT = vtype<decltype(fp)>;
                 for (int sw = 1; sw < h->o.nu_pre; sw++) {
                     A* xo = xcur[l];
                     A* xn = xalt[l];
-                    with_rpw(rpw, [&](auto R) {
+                    with_rpw<M>(rpw, [&](auto R) {
                         launch_pdl(k_sweep<decltype(R)::value, A, M, FT>, nb, kBlock, 0, s,
                             n, mat, fp, xo, Vw::invd(F), xn, st);
                     });
@@ -672,24 +703,24 @@ static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s) {
                 const A* xc = xcur[l];
                 if (l == 0) prof_mark(h, 1, 0, s);
                 if constexpr (std::is_same_v<A, double>) {
-                    if (l == 0 && h->sell64) {
+                    if (l == 0 && h->sell64 && !rows_only) {
                         sell64_resid(h, h->r, xc, rb, s);
                         prof_mark(h, 1, 1, s);
                         return;
                     }
                 }
                 if constexpr (std::is_same_v<A, float>) {
-                    if (l == 0 && h->stream) {
+                    if (l == 0 && h->stream && !rows_only) {
                         launch_stream_resid(h, h->r, xc, rb, s);
                         prof_mark(h, 1, 1, s);
                         return;
                     }
-                    if (l == 1 && h->sell[1].on) {
+                    if (l == 1 && h->sell[1].on && !rows_only) {
                         sell_resid1(h, static_cast<const float*>(Vw::f(F)), xc, rb, s);
                         return;
                     }
                 }
-                with_rpw(rpw, [&](auto R) {
+                with_rpw<M>(rpw, [&](auto R) {
                     launch_pdl(k_resid<decltype(R)::value, A, M, FT, A>, nb, kBlock, 0, s, n, mat, fp, xc, rb, st);
                 });
                 if (l == 0) prof_mark(h, 1, 1, s);
@@ -710,15 +741,15 @@ static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s) {
     for (int l = L - 2; l >= 0; l--) {
         Level& F = h->lev[l];
         const int n = F.A.n;
-        const int rpw = rows_per_warp(n, sms), nb = row_blocks(n, rpw);
-        Vw::vals(F, l, [&](auto mat) {
+        const int rpw = level_rows(h, F, rows_only), nb = row_blocks(n, rpw);
+        Vw::vals(F, l, rpw, [&](auto mat) {
             using M = decltype(mat);
             auto sweeps = [&](auto fp) {
                 using FT = vtype<decltype(fp)>;
                 for (int sw = 1; sw < h->o.nu_post; sw++) {
                     A* xo = xcur[l];
                     A* xn = xalt[l];
-                    with_rpw(rpw, [&](auto R) {
+                    with_rpw<M>(rpw, [&](auto R) {
                         launch_pdl(k_sweep<decltype(R)::value, A, M, FT>, nb, kBlock, 0, s,
                             n, mat, fp, xo, Vw::invd(F), xn, st);
                     });
@@ -732,30 +763,31 @@ static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s) {
             if (l == 0) {
                 prof_mark(h, 2, 0, s);
                 if constexpr (std::is_same_v<A, double>) {
-                    if (h->sell64) {
+                    if (h->sell64 && !rows_only) {
                         sell64_up0(h, h->r, xc, Vw::invd(F), h->z, h->q, slot(h, S_RZ), slot(h, S_ZQ), flex, s);
                         prof_mark(h, 2, 1, s);
                         return;
                     }
                 }
                 if constexpr (std::is_same_v<A, float>) {
-                    if (h->stream) {
+                    if (h->stream && !rows_only) {
                         launch_stream_up0(h, h->r, xc, Vw::invd(F), h->z, h->q, slot(h, S_RZ), slot(h, S_ZQ), flex,
                                           s);
                         prof_mark(h, 2, 1, s);
                         return;
                     }
                 }
-                with_rpw(rpw, [&](auto R) {
+                double* part_rz = rows_only ? nullptr : slot(h, S_RZ);
+                with_rpw<M>(rpw, [&](auto R) {
                     launch_pdl(k_up0<decltype(R)::value, A, M>, nb, kBlock, 0, s,
-                        n, mat, h->r, xc, Vw::invd(F), h->z, h->q, slot(h, S_RZ), slot(h, S_ZQ), flex, st);
+                        n, mat, h->r, xc, Vw::invd(F), h->z, h->q, part_rz, slot(h, S_ZQ), flex, st);
                 });
                 prof_mark(h, 2, 1, s);
             } else {
                 Level& G = h->lev[l - 1];
                 A* xf = xcur[l - 1];
                 if constexpr (std::is_same_v<A, float>) {
-                    if (l == 1 && h->sell[1].on) {  // y = smoothed level 1, then the gather into level 0
+                    if (l == 1 && h->sell[1].on && !rows_only) {  // y = smoothed level 1, then the gather into level 0
                         A* y = xalt[1];
                         sell_upy1(h, static_cast<const float*>(Vw::f(F)), xc, Vw::invd(F), y, s);
                         if (G.smoothed)
@@ -768,16 +800,16 @@ static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s) {
                 }
                 if (G.smoothed) {  // y = x + (f - K x) / d, then x_f += P_bar y
                     A* y = xalt[l];
-                    with_rpw(rpw, [&](auto R) {
+                    with_rpw<M>(rpw, [&](auto R) {
                         launch_pdl(k_sweep<decltype(R)::value, A, M, A>, nb, kBlock, 0, s, n, mat,
                                    static_cast<const A*>(Vw::f(F)), xc, Vw::invd(F), y, st);
                     });
                     sp_prolong<A>(G, y, xf, st, s);
                     return;
                 }
-                with_rpw(rpw, [&](auto R) {
+                with_rpw<M>(rpw, [&](auto R) {
                     launch_pdl(k_up<decltype(R)::value, A, M>, nb, kBlock, 0, s,
-                        n, mat, Vw::f(F), xc, Vw::invd(F), G.mem_ptr, G.mem_idx, G.pval, xf, st);
+                        n, mat, Vw::f(F), xc, Vw::invd(F), G.mem_ptr, G.mem_idx, G.agg, G.pval, xf, st);
                 });
             }
         });
@@ -810,7 +842,7 @@ static cudaError_t vcycle_cheb(amg_hierarchy* h, cudaStream_t s) {
         Level& F = h->lev[l];
         Level& C = h->lev[l + 1];
         const int n = F.A.n;
-        const int rpw = rows_per_warp(n, sms), nb = row_blocks(n, rpw), nv = vec_blocks(n, sms);
+        const int rpw = level_rows(h, F, false), nb = row_blocks(n, rpw), nv = vec_blocks(n, sms);
         A* x = Vw::x(F);
         A* r = Vw::t(F);
         A* d0 = static_cast<A*>(F.cd[0]);
@@ -818,12 +850,12 @@ static cudaError_t vcycle_cheb(amg_hierarchy* h, cudaStream_t s) {
         auto run = [&](auto fp) {
             using FT = vtype<decltype(fp)>;
             launch_pdl(k_cheb_start<A, FT>, nv, kBlock, 0, s, n, fp, Vw::invd(F), c0, x, d0, st);
-            Vw::vals(F, l, [&](auto mat) {
+            Vw::vals(F, l, rpw, [&](auto mat) {
                 using M = decltype(mat);
                 A* dp = d0;
                 A* dn = d1;
                 for (int i = 1; i < k; i++) {
-                    with_rpw(rpw, [&](auto R) {
+                    with_rpw<M>(rpw, [&](auto R) {
                         if (i == 1)
                             launch_pdl(k_cheb_step<decltype(R)::value, A, M, FT>, nb, kBlock, 0, s, n, mat,
                                        static_cast<const A*>(dp), fp, r, Vw::invd(F), coef_a(i), coef_b(i), dn, x,
@@ -835,7 +867,7 @@ static cudaError_t vcycle_cheb(amg_hierarchy* h, cudaStream_t s) {
                     });
                     std::swap(dp, dn);
                 }
-                with_rpw(rpw, [&](auto R) {
+                with_rpw<M>(rpw, [&](auto R) {
                     if (k == 1)
                         launch_pdl(k_cheb_resid<decltype(R)::value, A, M, FT>, nb, kBlock, 0, s, n, mat,
                                    static_cast<const A*>(dp), fp, r, x, st);
@@ -876,7 +908,7 @@ static cudaError_t vcycle_cheb(amg_hierarchy* h, cudaStream_t s) {
     for (int l = L - 2; l >= 0; l--) {
         Level& F = h->lev[l];
         const int n = F.A.n;
-        const int rpw = rows_per_warp(n, sms), nb = row_blocks(n, rpw), nv = vec_blocks(n, sms);
+        const int rpw = level_rows(h, F, false), nb = row_blocks(n, rpw), nv = vec_blocks(n, sms);
         A* x = Vw::x(F);
         A* r = Vw::t(F);
         A* d0 = static_cast<A*>(F.cd[0]);
@@ -884,16 +916,16 @@ static cudaError_t vcycle_cheb(amg_hierarchy* h, cudaStream_t s) {
         A* dlast = d0;
         auto run = [&](auto fp) {
             using FT = vtype<decltype(fp)>;
-            Vw::vals(F, l, [&](auto mat) {
+            Vw::vals(F, l, rpw, [&](auto mat) {
                 using M = decltype(mat);
-                with_rpw(rpw, [&](auto R) {
+                with_rpw<M>(rpw, [&](auto R) {
                     launch_pdl(k_cheb_post0<decltype(R)::value, A, M, FT>, nb, kBlock, 0, s, n, mat, fp,
                                static_cast<const A*>(x), Vw::invd(F), c0, r, d0, st);
                 });
                 A* dp = d0;
                 A* dn = d1;
                 for (int i = 1; i < k; i++) {
-                    with_rpw(rpw, [&](auto R) {
+                    with_rpw<M>(rpw, [&](auto R) {
                         launch_pdl(k_cheb_step<decltype(R)::value, A, M, A>, nb, kBlock, 0, s, n, mat,
                                    static_cast<const A*>(dp), static_cast<const A*>(r), r, Vw::invd(F), coef_a(i),
                                    coef_b(i), dn, x, st);
@@ -922,7 +954,7 @@ static cudaError_t vcycle_cheb(amg_hierarchy* h, cudaStream_t s) {
             else run(static_cast<const A*>(Vw::f(F)));
         }
         if (l == 0) {
-            const int nbz0 = (h->stream || h->sell64) ? h->stream_blocks : row_blocks(n, rows_per_warp(n, sms));
+            const int nbz0 = (h->stream || h->sell64) ? h->stream_blocks : row_blocks(n, rpw);
             launch_pdl(k_cheb_z<A>, nbz0, kBlock, 0, s, n, static_cast<const A*>(x), static_cast<const A*>(dlast),
                        static_cast<const double*>(h->r), h->z, static_cast<const double*>(h->q), slot(h, S_RZ),
                        slot(h, S_ZQ), flex, st);
@@ -944,9 +976,14 @@ cudaError_t enqueue_vcycle(amg_hierarchy* h, cudaStream_t s) {
     return h->mixed ? vcycle_impl<float>(h, s) : vcycle_impl<double>(h, s);
 }
 
+cudaError_t enqueue_vcycle_rows(amg_hierarchy* h, cudaStream_t s) {
+    return h->mixed ? vcycle_impl<float>(h, s, true) : vcycle_impl<double>(h, s, true);
+}
+
 // blocks of the level-0 row kernels, of the vector kernels, and of the
 // kernel that produces z (level-0 up sweep or single-level coarse solve)
-static int nb0(amg_hierarchy* h) { return row_blocks(h->lev[0].A.n, rows_per_warp(h->lev[0].A.n, h->num_sms)); }
+static int rows0(amg_hierarchy* h) { return level_rows(h, h->lev[0], false); }
+static int nb0(amg_hierarchy* h) { return row_blocks(h->lev[0].A.n, rows0(h)); }
 static int nbv(amg_hierarchy* h) { return vec_blocks(h->lev[0].A.n, h->num_sms); }
 // blocks (= partial sums) of the FP64 residual kernel
 static int nb_res(amg_hierarchy* h) {
@@ -958,7 +995,8 @@ static int nb_fine(amg_hierarchy* h) { return (h->stream || h->sell64) ? h->stre
 static int nbz(amg_hierarchy* h) { return h->nlev > 1 ? nb_fine(h) : row_blocks(h->ndense, 1); }
 
 size_t partial_slot_size(int n0, int num_sms) {
-    const int a = row_blocks(n0, rows_per_warp(n0, num_sms));
+    // the row-group kernels' fewest rows per warp (level_rows)
+    const int a = row_blocks(n0, rows_per_warp(n0, num_sms) == 8 ? 4 : 1);
     const int b = vec_blocks(n0, num_sms);
     const int m = a > b ? a : b;
     return (size_t)((m > num_sms ? m : num_sms) + 2);
@@ -972,13 +1010,13 @@ static cudaError_t launch_residual(amg_hierarchy* h, double* r, bool want_x0, in
                                    const SolveState* gate, cudaStream_t s) {
     Level& L0 = h->lev[0];
     const int n = L0.A.n;
-    const int rpw = rows_per_warp(n, h->num_sms), nb = nb_res(h);
+    const int rpw = rows0(h), nb = nb_res(h);
     const bool x0 = want_x0 && h->nlev > 1;
     double* pff = ff ? slot(h, S_FF) : nullptr;
-    with_rpw(rpw, [&](auto R) {
-        constexpr int RPW = decltype(R)::value;
-        with_mat(L0, static_cast<const double*>(L0.A.val), [&](auto mat) {
-            using M = decltype(mat);
+    with_mat(L0, static_cast<const double*>(L0.A.val), rpw, [&](auto mat) {
+        using M = decltype(mat);
+        with_rpw<M>(rpw, [&](auto R) {
+            constexpr int RPW = decltype(R)::value;
             if (h->mixed)
                 launch_pdl(k_residual0<RPW, float, M>, nb, kBlock, 0, s, n, mat, h->x, h->F, L0.invd32, r,
                                                                            x0 ? L0.x32 : nullptr, slot(h, rr_slot),
@@ -1013,25 +1051,28 @@ cudaError_t enqueue_pcg_iteration(amg_hierarchy* h, cudaStream_t s) {
     Level& L0 = h->lev[0];
     const int n = L0.A.n;
     const int flex = h->o.flexible;
-    const int rpw = rows_per_warp(n, h->num_sms), nb = row_blocks(n, rpw);
+    const int rpw = rows0(h), nb = row_blocks(n, rpw);
     prof_mark(h, 0, 0, s);
-    with_rpw(rpw, [&](auto R) {
-        constexpr int RPW = decltype(R)::value;
-        if (h->mixed && h->stream)
-            launch_stream_spmv_pq(h, h->p32, h->p, h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, s);
-        else if (h->sell64)
-            sell64_spmv_pq(h, h->p, h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, s);
-        else if (h->mixed)
-            with_mat(L0, static_cast<const float*>(L0.val32), [&](auto mat) {
-                launch_pdl(k_spmv_pq<RPW, float, decltype(mat), float>, nb, kBlock, 0, s,
-                    n, mat, h->p32, h->p, h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, h->st);
+    if (h->mixed && h->stream)
+        launch_stream_spmv_pq(h, h->p32, h->p, h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, s);
+    else if (h->sell64)
+        sell64_spmv_pq(h, h->p, h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, s);
+    else if (h->mixed)
+        with_mat(L0, static_cast<const float*>(L0.val32), rpw, [&](auto mat) {
+            using M = decltype(mat);
+            with_rpw<M>(rpw, [&](auto R) {
+                launch_pdl(k_spmv_pq<decltype(R)::value, float, M, float>, nb, kBlock, 0, s, n, mat, h->p32, h->p,
+                           h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, h->st);
             });
-        else
-            with_mat(L0, static_cast<const double*>(L0.A.val), [&](auto mat) {
-                launch_pdl(k_spmv_pq<RPW, double, decltype(mat), double>, nb, kBlock, 0, s,
-                    n, mat, h->p, h->p, h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, h->st);
+        });
+    else
+        with_mat(L0, static_cast<const double*>(L0.A.val), rpw, [&](auto mat) {
+            using M = decltype(mat);
+            with_rpw<M>(rpw, [&](auto R) {
+                launch_pdl(k_spmv_pq<decltype(R)::value, double, M, double>, nb, kBlock, 0, s, n, mat, h->p, h->p,
+                           h->r, h->q, slot(h, S_PQ), slot(h, S_PR), flex, h->st);
             });
-    });
+        });
     prof_mark(h, 0, 1, s);
     launch_pdl(k_scal_alpha, 1, 256, 0, s, slot(h, S_PQ), slot(h, S_PR), nb_fine(h), flex, h->st);
     const bool x0 = h->nlev > 1;
@@ -1054,24 +1095,29 @@ cudaError_t enqueue_pcg_iteration(amg_hierarchy* h, cudaStream_t s) {
 }
 
 // The row-group q = K p pass of the finest level (the layout used when no
-// sliced or staged copy is in use), for the setup's autotuning.
-cudaError_t launch_rowgroup_pq(amg_hierarchy* h, cudaStream_t s) {
+// sliced or staged copy is in use), for the setup's autotuning and (without
+// the partial sums) for batches.
+cudaError_t launch_rowgroup_pq(amg_hierarchy* h, cudaStream_t s, bool batch) {
     Level& L0 = h->lev[0];
     const int n = L0.A.n;
-    const int rpw = rows_per_warp(n, h->num_sms), nb = row_blocks(n, rpw);
-    with_rpw(rpw, [&](auto R) {
-        constexpr int RPW = decltype(R)::value;
-        if (h->mixed)
-            with_mat(L0, static_cast<const float*>(L0.val32), [&](auto mat) {
-                launch_pdl(k_spmv_pq<RPW, float, decltype(mat), float>, nb, kBlock, 0, s, n, mat, h->p32, h->p,
-                           h->r, h->q, slot(h, S_PQ), slot(h, S_PR), 0, h->st);
+    const int rpw = level_rows(h, L0, batch), nb = row_blocks(n, rpw);
+    double* part_pq = batch ? nullptr : slot(h, S_PQ);
+    if (h->mixed)
+        with_mat(L0, static_cast<const float*>(L0.val32), rpw, [&](auto mat) {
+            using M = decltype(mat);
+            with_rpw<M>(rpw, [&](auto R) {
+                launch_pdl(k_spmv_pq<decltype(R)::value, float, M, float>, nb, kBlock, 0, s, n, mat, h->p32, h->p,
+                           h->r, h->q, part_pq, slot(h, S_PR), 0, h->st);
             });
-        else
-            with_mat(L0, static_cast<const double*>(L0.A.val), [&](auto mat) {
-                launch_pdl(k_spmv_pq<RPW, double, decltype(mat), double>, nb, kBlock, 0, s, n, mat, h->p, h->p,
-                           h->r, h->q, slot(h, S_PQ), slot(h, S_PR), 0, h->st);
+        });
+    else
+        with_mat(L0, static_cast<const double*>(L0.A.val), rpw, [&](auto mat) {
+            using M = decltype(mat);
+            with_rpw<M>(rpw, [&](auto R) {
+                launch_pdl(k_spmv_pq<decltype(R)::value, double, M, double>, nb, kBlock, 0, s, n, mat, h->p, h->p,
+                           h->r, h->q, part_pq, slot(h, S_PR), 0, h->st);
             });
-    });
+        });
     return cudaGetLastError();
 }
 
