@@ -858,8 +858,6 @@ void free_multi(amg_hierarchy* h) {
     if (!w) return;
     if (w->graph) cudaGraphExecDestroy(w->graph);
     for (void* p : w->allocs) cudaFreeAsync(p, h->s);
-    if (w->st_host) cudaFreeHost(w->st_host);
-    if (w->active_host) cudaFreeHost(w->active_host);
     delete w;
     h->mw = nullptr;
 }
@@ -1239,48 +1237,71 @@ int amg_pcg_solve(amg_hierarchy* h, const double* F, double* u, int32_t mem, dou
 }
 
 // ------------------------------------------------------ multi-system solves
-// Workspace for S systems over R interleaved vectors (reused when unchanged).
-static int ensure_multi(amg_hierarchy* h, int R, int S, const int32_t* seg, const int64_t* segoff) {
+// Workspace for S systems (reused when unchanged): R interleaved right-hand
+// sides, or (seg given) a batch's row tiles over the hierarchy's own vectors.
+static int ensure_multi(amg_hierarchy* h, int R, int S, const int32_t* seg) {
     if (h->mw && h->mw->R == R && h->mw->S == S && h->mw->seg == seg) return AMG_OK;
     CK(cudaStreamSynchronize(h->s));
     free_multi(h);
     MultiWork* w = new (std::nothrow) MultiWork();
     if (!w) return AMG_ERR_NOMEM;
     h->mw = w;
-    w->R = R;
-    w->Rp = pow2ceil(R);
     w->S = S;
     w->seg = seg;
-    w->segoff = segoff;
-    const size_t E = (size_t)h->lev[0].A.n * R;
-    RC(walloc(h, *w, &w->x, E));
-    RC(walloc(h, *w, &w->r, E));
-    RC(walloc(h, *w, &w->p, E));
-    RC(walloc(h, *w, &w->q, E));
-    RC(walloc(h, *w, &w->z, E));
-    RC(walloc(h, *w, &w->F, E));
-    RC(walloc(h, *w, &w->pa, E));
-    RC(walloc(h, *w, &w->pb, E));
-    RC(walloc(h, *w, &w->stage, E));
-    if (h->mixed) RC(walloc(h, *w, &w->p32, E));
-    RC(walloc(h, *w, &w->dots, (size_t)S * multi_dot_stride()));
+    if (seg) {
+        // tiles of at most kTileRows rows of one system
+        constexpr int64_t kTileRows = 1024;
+        std::vector<int4> tiles;
+        std::vector<int> tile0(S + 1, 0);
+        for (int k = 0; k < S; k++) {
+            for (int64_t r = h->sys_off[k]; r < h->sys_off[k + 1]; r += kTileRows)
+                tiles.push_back(make_int4(k, (int)r, (int)std::min(r + kTileRows, h->sys_off[k + 1]), 0));
+            tile0[k + 1] = (int)tiles.size();
+        }
+        w->ntiles = (int)tiles.size();
+        RC(walloc(h, *w, &w->tiles, tiles.size()));
+        RC(walloc(h, *w, &w->tile0, tile0.size()));
+        CK(cudaMemcpyAsync(w->tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, h->s));
+        CK(cudaMemcpyAsync(w->tile0, tile0.data(), sizeof(int) * tile0.size(), cudaMemcpyHostToDevice, h->s));
+        CK(cudaStreamSynchronize(h->s));  // the host arrays end here
+        w->x = h->x;
+        w->r = h->r;
+        w->p = h->p;
+        w->q = h->q;
+        w->z = h->z;
+        w->F = h->F;
+        w->p32 = h->p32;
+    } else {
+        w->Rs = (R + 3) & ~3;
+        const size_t E = (size_t)h->lev[0].A.n * w->Rs;
+        for (double** v : {&w->x, &w->r, &w->p, &w->q, &w->z, &w->F}) {
+            RC(walloc(h, *w, v, E));
+            CK(cudaMemsetAsync(*v, 0, sizeof(double) * E, h->s));
+        }
+        RC(walloc(h, *w, &w->stage, (size_t)h->lev[0].A.n * R));
+        if (h->mixed) {
+            RC(walloc(h, *w, &w->p32, E));
+            CK(cudaMemsetAsync(w->p32, 0, sizeof(float) * E, h->s));
+        }
+        for (int l = 0; l < h->nlev; l++) {
+            const size_t El = (size_t)h->lev[l].A.n * w->Rs * (h->mixed ? 4 : 8);
+            for (void** v : {&w->lf[l], &w->lx[l], &w->lt[l]}) {
+                if (v == &w->lf[l] && l == 0) continue;  // level 0's right-hand side is r
+                char* b = nullptr;
+                RC(walloc(h, *w, &b, El));
+                CK(cudaMemsetAsync(b, 0, El, h->s));
+                *v = b;
+            }
+        }
+    }
+    w->part_stride = multi_part_stride(h, w->Rs, w->ntiles);
+    RC(walloc(h, *w, &w->part, w->part_stride * multi_part_slots()));
+    RC(walloc(h, *w, &w->dots, (size_t)S * 2));
     RC(walloc(h, *w, &w->st, (size_t)S));
     RC(walloc(h, *w, &w->active, 1));
     RC(walloc(h, *w, &w->params, 2));
-    CK(cudaMemsetAsync(w->pb, 0, sizeof(double) * E, h->s));
-    for (int l = 0; l < h->nlev; l++) {
-        const size_t El = (size_t)h->lev[l].A.n * R;
-        const size_t b = h->mixed ? 4 : 8;
-        char *f = nullptr, *x = nullptr, *t = nullptr;
-        if (l > 0) RC(walloc(h, *w, &f, El * b));
-        RC(walloc(h, *w, &x, El * b));
-        RC(walloc(h, *w, &t, El * b));
-        w->lf[l] = f;
-        w->lx[l] = x;
-        w->lt[l] = t;
-    }
-    CK(cudaMallocHost(&w->st_host, sizeof(MultiState) * S));
-    CK(cudaMallocHost(&w->active_host, sizeof(int)));
+    RC(walloc(h, *w, &w->due, 1));
+    w->R = R;  // complete: a failed attempt is built again
     return AMG_OK;
 }
 
@@ -1311,26 +1332,27 @@ static int run_multi(amg_hierarchy* h, int32_t* iters, double* relres, int32_t* 
     }
     const int max_launches = h->itmax / kGraphIters + 2;
     for (int k = 0; k <= max_launches + 1; k++) {
-        CK(cudaMemcpyAsync(w.active_host, w.active, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(h->flag_host, w.active, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        if (*w.active_host == 0 || k > max_launches) break;
+        if (*h->flag_host == 0 || k > max_launches) break;
         CK(cudaGraphLaunch(w.graph, s));
         amg::g_launches += w.graph_kernels;
     }
     CK(cudaEventRecord(h->ev1, s));
     CK(enqueue_multi_final(h, s));
-    std::vector<double> dots((size_t)w.S * multi_dot_stride());
+    std::vector<double> dots((size_t)w.S * 2);
     CK(cudaMemcpyAsync(dots.data(), w.dots, sizeof(double) * dots.size(), cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(w.st_host, w.st, sizeof(MultiState) * w.S, cudaMemcpyDeviceToHost, s));
+    std::vector<MultiState> states(w.S);
+    CK(cudaMemcpyAsync(states.data(), w.st, sizeof(MultiState) * w.S, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, h->ev0, h->ev1);
     h->info.solve_ms = ms;
     int worst = AMG_OK, maxit = 0;
     for (int k = 0; k < w.S; k++) {
-        const MultiState& m = w.st_host[k];
-        const double rr = std::sqrt(dots[(size_t)k * multi_dot_stride() + 0]);
-        const double ff = std::sqrt(dots[(size_t)k * multi_dot_stride() + 1]);
+        const MultiState& m = states[k];
+        const double rr = std::sqrt(dots[(size_t)k * 2]);
+        const double ff = std::sqrt(dots[(size_t)k * 2 + 1]);
         int st = m.done ? m.status : AMG_ERR_NOT_CONVERGED;
         if (iters) iters[k] = m.iters;
         if (relres) relres[k] = (ff > 0.0 && m.nF > 0.0) ? rr / ff : 0.0;
@@ -1362,18 +1384,18 @@ int amg_pcg_solve_multi(amg_hierarchy* h, int32_t nrhs, const double* F, double*
     if (ld < n) return AMG_ERR_ARG;
     RC(check_multi_opts(h));
     RC(join_caller(h));
-    RC(ensure_multi(h, nrhs, nrhs, nullptr, nullptr));
+    RC(ensure_multi(h, nrhs, nrhs, nullptr));
     MultiWork& w = *h->mw;
     cudaStream_t s = h->s;
     const size_t colb = sizeof(double) * n, ldb = sizeof(double) * ld;
     if (mem == AMG_MEM_HOST) {
         CK(cudaMemcpy2DAsync(w.stage, colb, F, ldb, colb, nrhs, cudaMemcpyHostToDevice, s));
-        CK(launch_interleave(n, nrhs, n, w.stage, w.F, s));
+        CK(launch_interleave(n, nrhs, w.Rs, n, w.stage, w.F, s));
         CK(cudaMemcpy2DAsync(w.stage, colb, U, ldb, colb, nrhs, cudaMemcpyHostToDevice, s));
-        CK(launch_interleave(n, nrhs, n, w.stage, w.x, s));
+        CK(launch_interleave(n, nrhs, w.Rs, n, w.stage, w.x, s));
     } else {
-        CK(launch_interleave(n, nrhs, ld, F, w.F, s));
-        CK(launch_interleave(n, nrhs, ld, U, w.x, s));
+        CK(launch_interleave(n, nrhs, w.Rs, ld, F, w.F, s));
+        CK(launch_interleave(n, nrhs, w.Rs, ld, U, w.x, s));
     }
     h->rtol = rtol;
     h->itmax = itmax;
@@ -1381,13 +1403,13 @@ int amg_pcg_solve_multi(amg_hierarchy* h, int32_t nrhs, const double* F, double*
     const int rc = run_multi(h, iters, relres, zero.data());
     if (rc == AMG_ERR_CUDA || rc == AMG_ERR_NOMEM) return rc;
     if (mem == AMG_MEM_HOST) {
-        CK(launch_deinterleave(n, nrhs, n, w.x, w.stage, s));
+        CK(launch_deinterleave(n, nrhs, w.Rs, n, w.x, w.stage, s));
         CK(cudaMemcpy2DAsync(U, ldb, w.stage, colb, colb, nrhs, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         for (int k = 0; k < nrhs; k++)
             if (zero[k]) memset(U + (size_t)k * ld, 0, colb);
     } else {
-        CK(launch_deinterleave(n, nrhs, ld, w.x, U, s));
+        CK(launch_deinterleave(n, nrhs, w.Rs, ld, w.x, U, s));
         for (int k = 0; k < nrhs; k++)
             if (zero[k]) CK(cudaMemsetAsync(U + (size_t)k * ld, 0, colb, s));
         CK(cudaStreamSynchronize(s));
@@ -1404,7 +1426,7 @@ int amg_pcg_solve_batch(amg_hierarchy* h, const double* const* F, double* const*
         if (!F[k] || !U[k]) return AMG_ERR_ARG;
     RC(check_multi_opts(h));
     RC(join_caller(h));
-    RC(ensure_multi(h, 1, h->nsys, h->sys_id, h->sys_off_dev));
+    RC(ensure_multi(h, 1, h->nsys, h->sys_id));
     MultiWork& w = *h->mw;
     cudaStream_t s = h->s;
     const cudaMemcpyKind in = mem == AMG_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;

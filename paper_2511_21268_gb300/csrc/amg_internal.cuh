@@ -48,21 +48,25 @@ struct MultiState {
     double nF, tol, rho, alpha, beta, pq, nr;
 };
 
-// Workspace of a multi-system solve.  Vectors are interleaved [N][R].
+// Workspace of a multi-system solve.  Several right-hand sides: vectors
+// interleaved [N][Rs], Rs = R rounded up to a multiple of 4.  Batch: the
+// hierarchy's own vectors, and the systems' rows in tiles.
 struct MultiWork {
-    int R = 0, Rp = 0, S = 0;
-    const int32_t* seg = nullptr;     // batch: system of each row (R = 1)
-    const int64_t* segoff = nullptr;  // batch: [S + 1] row offsets of the systems
+    int R = 0, Rs = 0, S = 0;
+    const int32_t* seg = nullptr;  // batch: system of each row (R = 1)
     double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *F = nullptr;
     float* p32 = nullptr;
-    double *pa = nullptr, *pb = nullptr;  // per-element products for the dots
-    double* dots = nullptr;               // [S][7]
-    double* stage = nullptr;              // column-major staging for copies
+    int4* tiles = nullptr;   // batch: (system, first row, end row) of each tile
+    int* tile0 = nullptr;    // batch: [S + 1] first tile of each system
+    int ntiles = 0;
+    double* part = nullptr;  // partial sums of two dot products
+    size_t part_stride = 0;
+    double* dots = nullptr;   // [S][2] final squared norms of F - K x and F
+    double* stage = nullptr;  // column-major staging for copies
     MultiState* st = nullptr;
-    MultiState* st_host = nullptr;
-    int* active = nullptr;     // systems still iterating
-    int* active_host = nullptr;
-    int* params = nullptr;     // itmax, replacement period
+    int* active = nullptr;    // systems still iterating
+    int* params = nullptr;    // itmax, replacement period
+    unsigned* due = nullptr;  // right-hand sides (batch: any) whose residual replacement is due
     void* lf[AMG_MAX_LEVELS] = {};
     void* lx[AMG_MAX_LEVELS] = {};
     void* lt[AMG_MAX_LEVELS] = {};
@@ -314,7 +318,8 @@ double* final_residual_slot(amg_hierarchy* h);
 cudaError_t enqueue_multi_start(amg_hierarchy* h, cudaStream_t s);
 cudaError_t enqueue_multi_iteration(amg_hierarchy* h, cudaStream_t s);
 cudaError_t enqueue_multi_final(amg_hierarchy* h, cudaStream_t s);
-int multi_dot_stride();
+size_t multi_part_stride(amg_hierarchy* h, int Rs, int ntiles);
+int multi_part_slots();
 // mpnn.cu
 void mpnn_free(amg_hierarchy* h);
 int mpnn_setup_fork(amg_hierarchy* h);
@@ -377,8 +382,8 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t s);
 // Records a CUDA error for amg_last_cuda_error; AMG_ERR_NOMEM for an
 // allocation failure, else AMG_ERR_CUDA.
 int report_cuda(cudaError_t e, const char* what);
-cudaError_t launch_interleave(int n, int R, int64_t ld, const double* src, double* dst, cudaStream_t s);
-cudaError_t launch_deinterleave(int n, int R, int64_t ld, const double* src, double* dst, cudaStream_t s);
+cudaError_t launch_interleave(int n, int R, int Rs, int64_t ld, const double* src, double* dst, cudaStream_t s);
+cudaError_t launch_deinterleave(int n, int R, int Rs, int64_t ld, const double* src, double* dst, cudaStream_t s);
 // batch assembly (setup_kernels.cu)
 cudaError_t launch_shift_block(int n, int64_t nnz, const int64_t* rp_in, int64_t row_off, int64_t nnz_off,
                                int64_t* rp_out, int32_t* col, int* flag, cudaStream_t s);

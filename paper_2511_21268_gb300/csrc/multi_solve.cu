@@ -2,288 +2,813 @@
 // run in one graph-captured loop (arXiv 2511.21268 Sec. 3 V-cycle and CG;
 // the batching is this library's design).
 //
-//   * R right-hand sides of one matrix: vectors interleaved as [N][R]; a
-//     matrix pass reads each matrix entry once for all R vectors (SpMM):
-//     R lanes (rounded up to a power of two) share a row, every lane owns
-//     one right-hand side, the entry value and column are broadcast and
-//     the R vector values of a column are one coalesced load.  System s =
-//     right-hand side s.
+//   * R right-hand sides of one matrix (k_m_*): vectors interleaved as
+//     [N][Rs], Rs = R rounded up to a multiple of 4, the padding columns
+//     zero; a matrix pass reads each matrix entry once for all R vectors
+//     (SpMM).  System s = right-hand side s.
 //   * a batch of independent matrices assembled block-diagonally into one
-//     hierarchy (there are no coupling entries, so matchings, aggregates and
-//     Galerkin products never cross blocks and every level operator is
-//     block diagonal): R = 1, system of row i = seg[i].
+//     hierarchy (k_b_*; there are no coupling entries, so matchings,
+//     aggregates and Galerkin products never cross blocks and every level
+//     operator is block diagonal): the V-cycle and q = K p are the
+//     single-system row-group kernels on the whole matrix, the vector
+//     kernels run on tiles of one system's rows each.
 //
 // Each system has its own CG scalars and convergence test; the dot products
-// are per-system sums in a fixed order (deterministic).  Converged systems
-// are frozen while the others iterate.  The V-cycle uses one pre- and one
-// post-smoothing sweep.
+// are per-system sums in a fixed order (deterministic): one partial sum per
+// block or tile, added up by the kernel that updates the scalars.  Converged
+// systems are frozen while the others iterate.  The V-cycle uses one pre-
+// and one post-smoothing sweep.
+//
+// What bounds the SpMM and why this split.  Per stored entry it needs the
+// entry's value and column and Rs vector values, one row of the interleaved
+// vector (64 bytes for 16 right-hand sides in FP32) gathered through L1.  A
+// lane owns 16 bytes of that row (4 right-hand sides in FP32, 2 in FP64), lp =
+// Rs sizeof / 16 lanes (rounded up to a power of two) cover it, and the warp's
+// 32 / lp lane groups take different entries, so that the value and column
+// loads are one wavefront for the whole group.  The gathers are bound by
+// their latency, so fewer of them is what helps: on the finest level the
+// run-encoded columns show which vector rows four neighbouring matrix rows
+// share (10 instead of 28 for runs of 7), and a warp takes four rows at once
+// (spmm_runs); the other levels go row by row (spmm_rows).  FP64 instructions
+// occupy GB300's two-lane FP64 pipe for 16 cycles however few lanes are
+// active, so the epilogues (FP64 dot products and conversions) run with a
+// (row, right-hand side) pair per lane, and the partial sums of a dot product
+// are few.  Measured, 3-D p = 3 n = 32 (10.5 M entries), 16 right-hand sides in
+// mixed precision, us per pass before (a lane per right-hand side, every entry
+// a load of its own) and after: q = K p 102 -> 58, residual 106 -> 67, up
+// sweep 100 -> 59, a level below the first 33 and 19 -> 11 and 10, the dots and
+// scalars of an iteration 140 -> 31; 102.5 -> 50.9 ms a solve.
+//
+// A batch's passes over level 0 (24 2-D systems, p 2..4, n 32..160, mixed
+// precision): 46, 40 and 35 us with a thread per row -> 27, 26 and 26 us with
+// the staged row order of CsrM::ordered; 42.5 -> 29.6 ms setup and solve.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "amg_internal.cuh"
+#include "row_kernels.cuh"
 
 namespace amg {
 
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
-enum { D_RR = 0, D_FF, D_PQ, D_PR, D_RZ, D_ZQ, D_RR2, D_COUNT };
+// ------------------------------------------------------ 16-byte vector access
+template <typename T>
+constexpr int kVec = 16 / sizeof(T);  // right-hand sides per lane
+template <typename T>
+constexpr int kBatch = sizeof(T) == 4 ? 8 : 4;  // entries per lane group in flight (row by row)
 
-__device__ __forceinline__ double ldm(const double* v, int64_t k) { return __ldg(v + k); }
-__device__ __forceinline__ float ldm(const float* v, int64_t k) { return __ldg(v + k); }
-__device__ __forceinline__ float ldm(const __nv_bfloat16* v, int64_t k) { return __bfloat162float(v[k]); }
-
-// Element (row i, vector c) handled by this thread; false when outside.
-#define MULTI_ELEM(n, R, Rp)                                      \
-    const int64_t g__ = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; \
-    const int i = (int)(g__ / (Rp)), c = (int)(g__ % (Rp));       \
-    if (i >= (n) || c >= (R)) return;
-
-__device__ __forceinline__ int sys_of(const int32_t* seg, int i, int c) { return seg ? seg[i] : c; }
-
-// sum_k v_k X[col_k][c] over row i (values V, vectors X, accumulation A)
-template <typename A, typename V, typename X>
-__device__ __forceinline__ A row_dot_m(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                       const V* __restrict__ v, const X* __restrict__ x, int i, int R, int c) {
-    const int64_t b = rp[i], e = rp[i + 1];
-    A acc = A(0);
-    int64_t k = b;
-    for (; k + 3 < e; k += 4) {
-        const A v0 = (A)ldm(v, k), v1 = (A)ldm(v, k + 1), v2 = (A)ldm(v, k + 2), v3 = (A)ldm(v, k + 3);
-        const int c0 = __ldg(ci + k), c1 = __ldg(ci + k + 1), c2 = __ldg(ci + k + 2), c3 = __ldg(ci + k + 3);
-        const A x0 = (A)x[(int64_t)c0 * R + c], x1 = (A)x[(int64_t)c1 * R + c];
-        const A x2 = (A)x[(int64_t)c2 * R + c], x3 = (A)x[(int64_t)c3 * R + c];
-        acc = fma(v0, x0, acc);
-        acc = fma(v1, x1, acc);
-        acc = fma(v2, x2, acc);
-        acc = fma(v3, x3, acc);
+// N consecutive values in 16-byte pieces (p aligned to 16 bytes)
+template <int N>
+__device__ __forceinline__ void load_vec(const float* __restrict__ p, float (&v)[N]) {
+    static_assert(N == 4, "a lane owns 4 FP32 columns");
+    const float4 a = *reinterpret_cast<const float4*>(p);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+}
+template <int N>
+__device__ __forceinline__ void load_vec(const double* __restrict__ p, double (&v)[N]) {
+    static_assert(N % 2 == 0, "16-byte pieces");
+#pragma unroll
+    for (int j = 0; j < N; j += 2) {
+        const double2 a = *reinterpret_cast<const double2*>(p + j);
+        v[j] = a.x, v[j + 1] = a.y;
     }
-    for (; k < e; k++) acc = fma((A)ldm(v, k), (A)x[(int64_t)__ldg(ci + k) * R + c], acc);
-    return acc;
+}
+// Lane layout of the SpMM kernels.  Gather: lane group g = lane / lp takes
+// every (32 / lp)-th entry, the lane's kVec columns start at c0.  After the
+// reduction a lane holds column c (own: c < Rs) of the row that its copy
+// index dup selects; 32 / (kVec lp) copies of each column.
+struct Lanes {
+    int lp, g, c0, c, dup;
+    bool own;
+};
+template <typename A>
+__device__ __forceinline__ Lanes lanes_of(int Rs, int lp) {
+    const int lane = threadIdx.x & 31, q = lane & (lp - 1);
+    Lanes L;
+    L.lp = lp;
+    L.g = lane / lp;
+    L.c0 = q * kVec<A> < Rs ? q * kVec<A> : 0;  // lanes past the last column repeat the first
+    if (kVec<A> == 4) {
+        L.c = q * 4 + ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
+        L.dup = (lane & 7) / lp;
+    } else {
+        L.c = q * 2 + ((lane >> 4) & 1);
+        L.dup = (lane & 15) / lp;
+    }
+    L.own = L.c < Rs;
+    return L;
+}
+template <typename A>
+__device__ __forceinline__ int copies_of(const Lanes& L) {
+    return 32 / (kVec<A> * L.lp);
 }
 
-// ----------------------------------------------------------------- kernels
-// FP64 residual r = F - K x; x0 = r / d (V-cycle precision); products r^2
-// and F^2.  gate: only systems whose replacement is due.
+// Sum over the lane groups; the lane's column c is returned (each step of
+// the first halves the columns a lane carries).
+__device__ __forceinline__ float reduce_columns(const float (&a)[4], const Lanes& L) {
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, e = lane & 8;
+    const float b0 = (h ? a[2] : a[0]) + __shfl_xor_sync(FULL, h ? a[0] : a[2], 16);
+    const float b1 = (h ? a[3] : a[1]) + __shfl_xor_sync(FULL, h ? a[1] : a[3], 16);
+    float s = (e ? b1 : b0) + __shfl_xor_sync(FULL, e ? b0 : b1, 8);
+    for (int o = 4; o >= L.lp; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+    return s;
+}
+__device__ __forceinline__ double reduce_columns(const double (&a)[2], const Lanes& L) {
+    const bool h = threadIdx.x & 16;
+    double s = (h ? a[1] : a[0]) + __shfl_xor_sync(FULL, h ? a[0] : a[1], 16);
+    for (int o = 8; o >= L.lp; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+    return s;
+}
+
+// acc[j] = sum_k v_k x[c_k][c0 + j] over the lane group's entries of a row of
+// `len` entries.  U vector rows per lane group are in flight; the values
+// and columns of the next batch load meanwhile.  Entries past the end are not
+// loaded (their product must not meet an infinite vector value).
+template <typename A, int U, typename V>
+__device__ __forceinline__ void row_dot(int len, const V* __restrict__ v, const int32_t* __restrict__ col,
+                                        const A* __restrict__ x, int Rs, const Lanes& L, A (&acc)[kVec<A>]) {
+    constexpr int N = kVec<A>;
+    const int G = 32 / L.lp;
+    const A* __restrict__ xc = x + L.c0;
+#pragma unroll
+    for (int j = 0; j < N; j++) acc[j] = A(0);
+    A vv[U], vn[U];
+    int cc[U], cn[U];
+    auto load = [&](int k, A (&vo)[U], int (&co)[U]) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const bool in = k + u * G < len;
+            vo[u] = in ? (A)ldv(v, k + u * G) : A(0);
+            co[u] = in ? __ldg(col + k + u * G) : -1;
+        }
+    };
+    load(L.g, vv, cc);
+    for (int k = 0; k < len; k += U * G) {  // warp-uniform
+        A xx[U][N];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (cc[u] >= 0) load_vec<N>(xc + (int64_t)cc[u] * Rs, xx[u]);
+        load(k + U * G + L.g, vn, cn);
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (cc[u] >= 0) {
+#pragma unroll
+                for (int j = 0; j < N; j++) acc[j] = fma(vv[u], xx[u][j], acc[j]);
+            }
+#pragma unroll
+        for (int u = 0; u < U; u++) vv[u] = vn[u], cc[u] = cn[u];
+    }
+    __syncwarp();
+}
+
+// Matrix views: plain CSR, and CSR with run-encoded columns as well.
+template <typename V>
+struct MatM {
+    const int64_t* __restrict__ rp;
+    const int32_t* __restrict__ ci;
+    const V* __restrict__ v;
+    const int32_t* __restrict__ rptr;  // null: no runs
+    const uint8_t* __restrict__ rlen;
+    const int32_t* __restrict__ rst;
+};
+
+// K x over the rows of this warp.  fin(i, valid, s) is called by all lanes
+// with the lane's row i, its column's sum s, and whether the lane has a (row,
+// column) pair at all.  Row by row: blocks of T consecutive rows (T at most
+// the copies of a column) share one call of fin.
+template <typename A, typename V, typename Fin>
+__device__ __forceinline__ void spmm_rows(int n, int Rs, int T, const Lanes& L, const MatM<V>& M,
+                                          const A* __restrict__ x, Fin&& fin) {
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, W = (gridDim.x * blockDim.x) >> 5;
+    for (int64_t i0 = (int64_t)warp * T; i0 < n; i0 += (int64_t)W * T) {
+        const int cnt = (int)min((int64_t)T, n - i0);
+        A keep = A(0);
+        for (int t = 0; t < cnt; t++) {
+            const int64_t b = M.rp[i0 + t];
+            A acc[kVec<A>];
+            row_dot<A, kBatch<A>>((int)(M.rp[i0 + t + 1] - b), M.v + b, M.ci + b, x, Rs, L, acc);
+            const A s = reduce_columns(acc, L);
+            if (L.dup == t) keep = s;
+        }
+        fin((int)i0 + L.dup, L.own && L.dup < cnt, keep);
+    }
+}
+
+// Four rows at once from the run-encoded columns.  In a tensor-product matrix
+// neighbouring rows of a line have the same number of runs, and run r of row
+// j starts delta_j columns after run r of the first row, delta_j the same for
+// all runs.  The lane groups take runs; per run the union of the four rows'
+// columns (W <= kRunSpan) is gathered once and multiplied into every row that
+// has the column.  Tiles that are not like that (the end of a line, any other
+// run structure, found while reading the runs) go row by row.
+constexpr int kTile = 4, kRunSpan = 12;
+template <typename A, typename V, typename Fin>
+__device__ __forceinline__ void spmm_runs(int n, int Rs, const Lanes& L, const MatM<V>& M, const A* __restrict__ x,
+                                          Fin&& fin) {
+    constexpr int N = kVec<A>, Q = 4;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, W = (gridDim.x * blockDim.x) >> 5;
+    const int G = 32 / L.lp, D = copies_of<A>(L);
+    const A* __restrict__ xc = x + L.c0;
+    for (int64_t i0 = (int64_t)warp * kTile; i0 < n; i0 += (int64_t)W * kTile) {
+        const int cnt = (int)min((int64_t)kTile, n - i0);
+        A acc[kTile][N];
+#pragma unroll
+        for (int j = 0; j < kTile; j++)
+#pragma unroll
+            for (int q = 0; q < N; q++) acc[j][q] = A(0);
+        bool ok = cnt == kTile;
+        if (ok) {
+            int rb[kTile], len[kTile], dl[kTile];
+            const V* vb[kTile];
+            const int runs = M.rptr[i0 + 1] - M.rptr[i0];
+            int span = 0;
+#pragma unroll
+            for (int j = 0; j < kTile; j++) {
+                rb[j] = M.rptr[i0 + j];
+                len[j] = M.rlen[i0 + j];
+                vb[j] = M.v + M.rp[i0 + j];
+                ok = ok && M.rptr[i0 + j + 1] - rb[j] == runs;
+            }
+            ok = ok && runs > 0;
+            if (ok) {
+                const int s0 = __ldg(M.rst + rb[0]);
+#pragma unroll
+                for (int j = 0; j < kTile; j++) {
+                    dl[j] = __ldg(M.rst + rb[j]) - s0;
+                    ok = ok && dl[j] >= 0 && dl[j] < kRunSpan;
+                    span = max(span, dl[j] + len[j]);
+                }
+                ok = ok && span <= kRunSpan;
+            }
+            if (ok) {  // uniform so far
+                bool same = true;
+                for (int r0 = 0; r0 < runs; r0 += G) {
+                    const int r = r0 + L.g;
+                    if (r < runs) {
+                        const int st = __ldg(M.rst + rb[0] + r);
+                        int vo[kTile];
+#pragma unroll
+                        for (int j = 0; j < kTile; j++) {
+                            if (j > 0) same = same && __ldg(M.rst + rb[j] + r) - st == dl[j];
+                            vo[j] = r * len[j] - dl[j];
+                        }
+#pragma unroll 1
+                        for (int o0 = 0; o0 < span; o0 += Q) {
+                            {
+                                A xx[Q][N], vv[kTile][Q];
+#pragma unroll
+                                for (int q = 0; q < Q; q++)
+                                    load_vec<N>(xc + (int64_t)min(st + min(o0 + q, span - 1), n - 1) * Rs, xx[q]);
+#pragma unroll
+                                for (int j = 0; j < kTile; j++)
+#pragma unroll
+                                    for (int q = 0; q < Q; q++) {
+                                        const bool in = (unsigned)(o0 + q - dl[j]) < (unsigned)len[j];
+                                        vv[j][q] = in ? (A)ldv(vb[j], vo[j] + o0 + q) : A(0);
+                                    }
+#pragma unroll
+                                for (int j = 0; j < kTile; j++)
+#pragma unroll
+                                    for (int q = 0; q < Q; q++)
+                                        if ((unsigned)(o0 + q - dl[j]) < (unsigned)len[j]) {
+#pragma unroll
+                                            for (int c = 0; c < N; c++)
+                                                acc[j][c] = fma(vv[j][q], xx[q][c], acc[j][c]);
+                                        }
+                            }
+                        }
+                    }
+                }
+                ok = __all_sync(FULL, same);
+            }
+        }
+        A s[kTile];
+        if (ok) {
+#pragma unroll
+            for (int j = 0; j < kTile; j++) s[j] = reduce_columns(acc[j], L);
+        } else {
+#pragma unroll 1
+            for (int t = 0; t < cnt; t++) {
+                const int64_t b = M.rp[i0 + t];
+                A a1[N];
+                row_dot<A, 4>((int)(M.rp[i0 + t + 1] - b), M.v + b, M.ci + b, x, Rs, L, a1);
+                const A r = reduce_columns(a1, L);
+#pragma unroll
+                for (int j = 0; j < kTile; j++)
+                    if (j == t) s[j] = r;
+            }
+        }
+        for (int base = 0; base < cnt; base += D) {
+            A keep = A(0);
+#pragma unroll
+            for (int j = 0; j < kTile; j++)
+                if (j == base + L.dup) keep = s[j];
+            fin((int)i0 + base + L.dup, L.own && base + L.dup < cnt, keep);
+        }
+    }
+}
+
+template <typename A, bool RUNS, typename V, typename Fin>
+__device__ __forceinline__ void spmm(int n, int Rs, int T, const Lanes& L, const MatM<V>& M, const A* __restrict__ x,
+                                     Fin&& fin) {
+    if constexpr (RUNS) spmm_runs<A>(n, Rs, L, M, x, fin);
+    else spmm_rows<A>(n, Rs, T, L, M, x, fin);
+}
+
+constexpr int kMaxRs = 32;  // padded right-hand sides
+
+// Block partial sums per right-hand side: every lane holds its column's sum;
+// *out receives Rs values (a column's copies, then the warps, in order).
+template <typename A>
+__device__ __forceinline__ void block_columns(double t, const Lanes& L, int Rs, double* sh, double* out) {
+    const int wid = threadIdx.x >> 5;
+    for (int o = (kVec<A> == 4 ? 4 : 8); o >= L.lp; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+    __syncthreads();
+    if (L.own && L.dup == 0) sh[wid * kMaxRs + L.c] = t;
+    __syncthreads();
+    if ((int)threadIdx.x < Rs) {
+        double s = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += sh[w * kMaxRs + threadIdx.x];
+        out[threadIdx.x] = s;
+    }
+}
+
+// Rows of a grid-stride kernel: a warp per row.
+#define SPMM_ROWS(i, n)                                                         \
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < (n);          \
+         i += (gridDim.x * blockDim.x) >> 5)
+
+// ------------------------------------------- kernels, several right-hand sides
+// FP64 residual r = F - K x; x0 = r / d (V-cycle precision); block partials
+// of r^2 and F^2.  due: only the right-hand sides of the mask (a residual
+// replacement); the kernel returns at once when it is empty.
 template <typename X0>
-__global__ void k_m_residual(int n, int R, int Rp, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                             const double* __restrict__ v, const double* __restrict__ x, const double* __restrict__ F,
-                             const X0* __restrict__ invd, double* r, X0* x0, double* pa, double* pb,
-                             const MultiState* gate, const int32_t* seg) {
-    MULTI_ELEM(n, R, Rp)
-    const int64_t e = (int64_t)i * R + c;
-    if (gate) {
-        const MultiState& s = gate[sys_of(seg, i, c)];
-        if (s.done || !s.replace_now) return;
-    }
-    const double fi = F[e];
-    const double ri = fi - row_dot_m<double>(rp, ci, v, x, i, R, c);
-    r[e] = ri;
-    if (x0) x0[e] = (X0)ri * invd[i];
-    pa[e] = ri * ri;
-    if (pb) pb[e] = fi * fi;
+__global__ void __launch_bounds__(kBlock, 2) k_m_residual(int n, int Rs, int lp, int T, MatM<double> mat,
+                                                        const double* __restrict__ x, const double* __restrict__ F,
+                                                        const X0* __restrict__ invd, double* r, X0* x0,
+                                                        double* part_rr, double* part_ff, const unsigned* due) {
+    pdl_entry();
+    const unsigned mask = due ? *due : FULL;
+    if (mask == 0) return;
+    __shared__ double sh[kWarpsPerBlock * kMaxRs];
+    const Lanes L = lanes_of<double>(Rs, lp);
+    double rr = 0.0, ff = 0.0;
+    const bool mine = L.own && (mask >> L.c & 1u);
+    spmm_rows<double>(n, Rs, T, L, mat, x, [&](int i, bool valid, double s) {
+        if (!valid || !mine) return;
+        const int64_t e = (int64_t)i * Rs + L.c;
+        const double fi = F[e], ri = fi - s;
+        r[e] = ri;
+        if (x0) x0[e] = (X0)ri * invd[i];
+        rr = fma(ri, ri, rr);
+        if (part_ff) ff = fma(fi, fi, ff);
+    });
+    block_columns<double>(rr, L, Rs, sh, part_rr + (int64_t)blockIdx.x * Rs);
+    if (part_ff) block_columns<double>(ff, L, Rs, sh, part_ff + (int64_t)blockIdx.x * Rs);
 }
 
-// Outer q = K p; products p.q and (flexible) p.r.
-template <typename A, typename V, typename PX>
-__global__ void k_m_spmv_pq(int n, int R, int Rp, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                            const V* __restrict__ v, const PX* __restrict__ pg, const double* __restrict__ p,
-                            const double* __restrict__ r, double* q, double* pa, double* pb, int flexible,
-                            const MultiState* st, const int32_t* seg, const int* active) {
+// Outer q = K p; block partials of p.q and (flexible) p.r.  The columns of
+// finished systems are computed too: nothing reads them.
+template <bool RUNS, typename A, typename V>
+__global__ void __launch_bounds__(kBlock, 2) k_m_spmv_pq(int n, int Rs, int lp, int T, MatM<V> mat,
+                                                       const A* __restrict__ pg, const double* __restrict__ p,
+                                                       const double* __restrict__ r, double* q, double* part_pq,
+                                                       double* part_pr, int flexible, const int* active) {
+    pdl_entry();
     if (*active == 0) return;
-    MULTI_ELEM(n, R, Rp)
-    if (st[sys_of(seg, i, c)].done) return;
-    const int64_t e = (int64_t)i * R + c;
-    const double qs = (double)row_dot_m<A>(rp, ci, v, pg, i, R, c);
-    q[e] = qs;
-    pa[e] = p[e] * qs;
-    if (flexible) pb[e] = p[e] * r[e];
+    __shared__ double sh[kWarpsPerBlock * kMaxRs];
+    const Lanes L = lanes_of<A>(Rs, lp);
+    double pq = 0.0, pr = 0.0;
+    spmm<A, RUNS>(n, Rs, T, L, mat, pg, [&](int i, bool valid, A s) {
+        if (!valid) return;
+        const int64_t e = (int64_t)i * Rs + L.c;
+        const double qs = (double)s, pi = p[e];
+        q[e] = qs;
+        pq = fma(pi, qs, pq);
+        if (flexible) pr = fma(pi, r[e], pr);
+    });
+    block_columns<A>(pq, L, Rs, sh, part_pq + (int64_t)blockIdx.x * Rs);
+    if (flexible) block_columns<A>(pr, L, Rs, sh, part_pr + (int64_t)blockIdx.x * Rs);
 }
 
 // V-cycle down-sweep residual rbuf = f - K x.
-template <typename A, typename V, typename FT>
-__global__ void k_m_resid(int n, int R, int Rp, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                          const V* __restrict__ v, const FT* __restrict__ f, const A* __restrict__ x, A* rbuf,
-                          const int* active) {
+template <bool RUNS, typename A, typename V, typename FT>
+__global__ void __launch_bounds__(kBlock, 2) k_m_resid(int n, int Rs, int lp, int T, MatM<V> mat,
+                                                     const FT* __restrict__ f, const A* __restrict__ x, A* rbuf,
+                                                     const int* active) {
+    pdl_entry();
     if (*active == 0) return;
-    MULTI_ELEM(n, R, Rp)
-    const int64_t e = (int64_t)i * R + c;
-    rbuf[e] = (A)f[e] - row_dot_m<A>(rp, ci, v, x, i, R, c);
+    const Lanes L = lanes_of<A>(Rs, lp);
+    spmm<A, RUNS>(n, Rs, T, L, mat, x, [&](int i, bool valid, A s) {
+        if (!valid) return;
+        const int64_t e = (int64_t)i * Rs + L.c;
+        rbuf[e] = (A)f[e] - s;
+    });
 }
 
 template <typename A>
-__global__ void k_m_restrict(int nc, int R, const int32_t* __restrict__ mptr, const int32_t* __restrict__ midx,
+__global__ void k_m_restrict(int nc, int Rs, const int32_t* __restrict__ mptr, const int32_t* __restrict__ midx,
                              const double* __restrict__ pval, const A* __restrict__ rbuf, A* fc, A* xc,
                              const A* __restrict__ invdc, const int* active) {
+    pdl_entry();
     if (*active == 0) return;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= (int64_t)nc * R) return;
-    const int I = (int)(g / R), c = (int)(g % R);
+    if (g >= (int64_t)nc * Rs) return;
+    const int I = (int)(g / Rs), c = (int)(g % Rs);
     A acc = A(0);
     for (int m = mptr[I]; m < mptr[I + 1]; m++) {
         const int a = midx[m];
-        acc = fma((A)pval[a], rbuf[(int64_t)a * R + c], acc);
+        acc = fma((A)pval[a], rbuf[(int64_t)a * Rs + c], acc);
     }
     fc[g] = acc;
     if (xc) xc[g] = acc * invdc[I];
 }
 
-// Coarsest level, e = A^-1 f per vector; prolongation into the finer level,
-// or (single-level hierarchy) z = e with the products r.z and z.q.
+// Coarsest level, e = A^-1 f per vector (FP64, a warp per row of the dense
+// inverse, one warp per block: the products spread over as many SMs' FP64
+// pipes as there are rows); prolongation into the finer level, or
+// (single-level hierarchy) z = e with the block partials of r.z and z.q.
+constexpr int kCoarseU = 8;  // entries of a lane group in flight
 template <typename FT, typename XT>
-__global__ void k_m_coarse(int nd, int R, const double* __restrict__ Ainv, const FT* __restrict__ f,
-                           const int32_t* __restrict__ mptr, const int32_t* __restrict__ midx,
-                           const double* __restrict__ pvalf, XT* xf, double* z, const double* __restrict__ q,
-                           double* pa, double* pb, int flexible, const int* active) {
+__global__ void __launch_bounds__(32) k_m_coarse(int nd, int Rs, int lp, const double* __restrict__ Ainv,
+                                                  const FT* __restrict__ f, const int32_t* __restrict__ mptr,
+                                                  const int32_t* __restrict__ midx,
+                                                  const double* __restrict__ pvalf, XT* xf, double* z,
+                                                  const double* __restrict__ q, double* part_rz, double* part_zq,
+                                                  int flexible, const int* active) {
+    pdl_entry();
     if (*active == 0) return;
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= (int64_t)nd * R) return;
-    const int I = (int)(g / R), c = (int)(g % R);
-    const double* row = Ainv + (int64_t)I * nd;
-    double s = 0.0;
-    for (int j = 0; j < nd; j++) s = fma(row[j], (double)f[(int64_t)j * R + c], s);
-    if (z) {
-        z[g] = s;
-        pa[g] = (double)f[g] * s;
-        if (flexible) pb[g] = s * q[g];
-    } else {
-        for (int m = mptr[I]; m < mptr[I + 1]; m++) {
-            const int a = midx[m];
-            const int64_t e = (int64_t)a * R + c;
-            xf[e] = (XT)fma(pvalf[a], s, (double)xf[e]);
-        }
-    }
-}
-
-template <typename A, typename V>
-__global__ void k_m_up(int n, int R, int Rp, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                       const V* __restrict__ v, const A* __restrict__ f, const A* __restrict__ x,
-                       const A* __restrict__ invd, const int32_t* __restrict__ mptr, const int32_t* __restrict__ midx,
-                       const double* __restrict__ pvalf, A* xf, const int* active) {
-    if (*active == 0) return;
-    MULTI_ELEM(n, R, Rp)
-    const int64_t e = (int64_t)i * R + c;
-    const A y = fma(invd[i], f[e] - row_dot_m<A>(rp, ci, v, x, i, R, c), x[e]);
-    for (int m = mptr[i]; m < mptr[i + 1]; m++) {
-        const int a = midx[m];
-        const int64_t ea = (int64_t)a * R + c;
-        xf[ea] = fma((A)pvalf[a], y, xf[ea]);
-    }
-}
-
-template <typename A, typename V>
-__global__ void k_m_up0(int n, int R, int Rp, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                        const V* __restrict__ v, const double* __restrict__ r, const A* __restrict__ x,
-                        const A* __restrict__ invd, double* z, const double* __restrict__ q, double* pa, double* pb,
-                        int flexible, const int* active) {
-    if (*active == 0) return;
-    MULTI_ELEM(n, R, Rp)
-    const int64_t e = (int64_t)i * R + c;
-    const double ra = r[e];
-    const double za = (double)fma(invd[i], (A)ra - row_dot_m<A>(rp, ci, v, x, i, R, c), x[e]);
-    z[e] = za;
-    pa[e] = ra * za;
-    if (flexible) pb[e] = za * q[e];
-}
-
-// x += alpha p, r -= alpha q, x0 = r / d, product r^2 (systems not done).
-template <typename X0>
-__global__ void k_m_update(int n, int R, double* x, double* r, const double* __restrict__ p,
-                           const double* __restrict__ q, const X0* __restrict__ invd, X0* x0, double* pa,
-                           const MultiState* st, const int32_t* seg, const int* active) {
-    if (*active == 0) return;
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= (int64_t)n * R) return;
-    const int i = (int)(g / R), c = (int)(g % R);
-    const MultiState& s = st[sys_of(seg, i, c)];
-    if (s.done) return;
-    const double alpha = s.alpha;
-    x[g] = fma(alpha, p[g], x[g]);
-    const double ri = fma(-alpha, q[g], r[g]);
-    r[g] = ri;
-    if (x0) x0[g] = (X0)ri * invd[i];
-    pa[g] = ri * ri;
-}
-
-__global__ void k_m_pupdate(int n, int R, double* p, const double* __restrict__ z, float* p32, int first,
-                            const MultiState* st, const int32_t* seg, const int* active) {
-    if (*active == 0) return;
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= (int64_t)n * R) return;
-    const int i = (int)(g / R), c = (int)(g % R);
-    const MultiState& s = st[sys_of(seg, i, c)];
-    if (s.done) return;
-    const double pi = first ? z[g] : fma(s.beta, p[g], z[g]);
-    p[g] = pi;
-    if (p32) p32[g] = __double2float_rn(pi);
-}
-
-// dots[s * D_COUNT + slot] = sum over the elements of system s (fixed order);
-// one block per system.
-__global__ void k_m_sys_sum(int n, int R, const int64_t* __restrict__ segoff, const double* __restrict__ pa, int sa,
-                            const double* __restrict__ pb, int sb, double* dots, const int* active) {
-    if (active && *active == 0) return;
-    const int s = blockIdx.x;
-    int64_t lo, hi, stride, off;
-    if (segoff) {
-        lo = segoff[s];
-        hi = segoff[s + 1];
-        stride = 1;
-        off = 0;
-    } else {
-        lo = 0;
-        hi = n;
-        stride = R;
-        off = s;
-    }
-    double a = 0.0, b = 0.0;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        a += pa[i * stride + off];
-        if (pb) b += pb[i * stride + off];
-    }
-    __shared__ double sha[32], shb[32];
+    __shared__ double sh[kMaxRs];
+    const Lanes L = lanes_of<double>(Rs, lp);
+    const int G = 32 / lp;
+    double rz = 0.0, zq = 0.0;
+    SPMM_ROWS(I, nd) {
+        const double* __restrict__ row = Ainv + (int64_t)I * nd;
+        double s2[2] = {0.0, 0.0};
+        for (int j0 = L.g; j0 < nd; j0 += kCoarseU * G) {
+            double a[kCoarseU], x0[kCoarseU], x1[kCoarseU];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(FULL, a, o);
-        b += __shfl_xor_sync(FULL, b, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        sha[threadIdx.x >> 5] = a;
-        shb[threadIdx.x >> 5] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-            ta += sha[w];
-            tb += shb[w];
+            for (int u = 0; u < kCoarseU; u++) {
+                const int j = j0 + u * G;
+                const bool in = j < nd;
+                const FT* fj = f + (int64_t)(in ? j : 0) * Rs + L.c0;
+                a[u] = in ? __ldg(row + j) : 0.0;
+                x0[u] = in ? (double)fj[0] : 0.0;
+                x1[u] = in ? (double)fj[1] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kCoarseU; u++) {
+                s2[0] = fma(a[u], x0[u], s2[0]);
+                s2[1] = fma(a[u], x1[u], s2[1]);
+            }
         }
-        dots[s * D_COUNT + sa] = ta;
-        if (pb) dots[s * D_COUNT + sb] = tb;
+        __syncwarp();
+        const double s = reduce_columns(s2, L);
+        if (z) {
+            if (L.own && L.dup == 0) {
+                const int64_t e = (int64_t)I * Rs + L.c;
+                z[e] = s;
+                rz = fma((double)f[e], s, rz);
+                if (flexible) zq = fma(s, q[e], zq);
+            }
+        } else if (L.own) {  // a member of the aggregate per copy of the column
+            const int m1 = mptr[I + 1], step = copies_of<double>(L);
+            for (int m = mptr[I] + L.dup; m < m1; m += step) {
+                const int a = midx[m];
+                XT* xe = xf + (int64_t)a * Rs + L.c;
+                *xe = (XT)fma(pvalf[a], s, (double)*xe);
+            }
+        }
+    }
+    if (z) {
+        block_columns<double>(rz, L, Rs, sh, part_rz + (int64_t)blockIdx.x * Rs);
+        if (flexible) block_columns<double>(zq, L, Rs, sh, part_zq + (int64_t)blockIdx.x * Rs);
+    }
+}
+
+// Up sweep of a level l >= 1: y = x + (f - K x) / d, prolongated into the
+// finer level.
+template <typename A, typename V>
+__global__ void __launch_bounds__(kBlock, 2) k_m_up(int n, int Rs, int lp, int T, MatM<V> mat,
+                                                  const A* __restrict__ f, const A* __restrict__ x,
+                                                  const A* __restrict__ invd, const int32_t* __restrict__ mptr,
+                                                  const int32_t* __restrict__ midx, const double* __restrict__ pvalf,
+                                                  A* xf, const int* active) {
+    pdl_entry();
+    if (*active == 0) return;
+    const Lanes L = lanes_of<A>(Rs, lp);
+    spmm_rows<A>(n, Rs, T, L, mat, x, [&](int i, bool valid, A s) {
+        if (!valid) return;
+        const int64_t e = (int64_t)i * Rs + L.c;
+        const A y = fma(invd[i], f[e] - s, x[e]);
+        const int m1 = mptr[i + 1];
+        for (int m = mptr[i]; m < m1; m++) {
+            const int a = midx[m];
+            A* xe = xf + (int64_t)a * Rs + L.c;
+            *xe = fma((A)pvalf[a], y, *xe);
+        }
+    });
+}
+
+// Up sweep of level 0: z = x + (r - K x) / d; block partials of r.z and
+// (flexible) z.q.
+template <bool RUNS, typename A, typename V>
+__global__ void __launch_bounds__(kBlock, 2) k_m_up0(int n, int Rs, int lp, int T, MatM<V> mat,
+                                                   const double* __restrict__ r, const A* __restrict__ x,
+                                                   const A* __restrict__ invd, double* z,
+                                                   const double* __restrict__ q, double* part_rz, double* part_zq,
+                                                   int flexible, const int* active) {
+    pdl_entry();
+    if (*active == 0) return;
+    __shared__ double sh[kWarpsPerBlock * kMaxRs];
+    const Lanes L = lanes_of<A>(Rs, lp);
+    double rz = 0.0, zq = 0.0;
+    spmm<A, RUNS>(n, Rs, T, L, mat, x, [&](int i, bool valid, A s) {
+        if (!valid) return;
+        const int64_t e = (int64_t)i * Rs + L.c;
+        const double ra = r[e];
+        const double za = (double)fma(invd[i], (A)ra - s, x[e]);
+        z[e] = za;
+        rz = fma(ra, za, rz);
+        if (flexible) zq = fma(za, q[e], zq);
+    });
+    block_columns<A>(rz, L, Rs, sh, part_rz + (int64_t)blockIdx.x * Rs);
+    if (flexible) block_columns<A>(zq, L, Rs, sh, part_zq + (int64_t)blockIdx.x * Rs);
+}
+
+// Threads of the vector kernels: Rs / 2 threads per row (two columns each),
+// kBlock / (Rs / 2) rows of a block at a time.
+struct PairLayout {
+    int lpr, rpb, rl, c;
+    bool in;
+};
+__device__ __forceinline__ PairLayout pair_layout(int Rs) {
+    PairLayout P;
+    P.lpr = Rs >> 1;
+    P.rpb = kBlock / P.lpr;
+    P.rl = threadIdx.x / P.lpr;
+    P.c = 2 * (threadIdx.x - P.rl * P.lpr);
+    P.in = P.rl < P.rpb;
+    return P;
+}
+
+// x += alpha p, r -= alpha q, x0 = r / d, block partials of r^2 (systems not
+// done).
+template <typename X0>
+__global__ void __launch_bounds__(kBlock) k_m_update(int n, int R, int Rs, double* x, double* r,
+                                                      const double* __restrict__ p, const double* __restrict__ q,
+                                                      const X0* __restrict__ invd, X0* x0, double* part_rr,
+                                                      const MultiState* st, const int* active) {
+    pdl_entry();
+    if (*active == 0) return;
+    __shared__ double sh[2 * kBlock];
+    const PairLayout P = pair_layout(Rs);
+    double rr[2] = {0.0, 0.0};
+    if (P.in) {
+        double alpha[2];
+        bool on[2];
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+            on[j] = P.c + j < R && !st[P.c + j].done;
+            alpha[j] = on[j] ? st[P.c + j].alpha : 0.0;
+        }
+        if (on[0] || on[1])
+            for (int64_t i = (int64_t)blockIdx.x * P.rpb + P.rl; i < n; i += (int64_t)gridDim.x * P.rpb) {
+                const int64_t e = i * Rs + P.c;
+                double xv[2], rv[2], pv[2], qv[2];
+                load_vec<2>(x + e, xv);
+                load_vec<2>(r + e, rv);
+                load_vec<2>(p + e, pv);
+                load_vec<2>(q + e, qv);
+                const X0 d = x0 ? invd[i] : X0(0);
+#pragma unroll
+                for (int j = 0; j < 2; j++) {
+                    if (!on[j]) continue;
+                    x[e + j] = fma(alpha[j], pv[j], xv[j]);
+                    const double ri = fma(-alpha[j], qv[j], rv[j]);
+                    r[e + j] = ri;
+                    if (x0) x0[e + j] = (X0)ri * d;
+                    rr[j] = fma(ri, ri, rr[j]);
+                }
+            }
+    }
+    sh[2 * threadIdx.x] = rr[0];
+    sh[2 * threadIdx.x + 1] = rr[1];
+    __syncthreads();
+    if ((int)threadIdx.x < Rs) {  // column c: its rows' threads in order
+        double s = 0.0;
+        for (int w = 0; w < P.rpb; w++) s += sh[w * Rs + threadIdx.x];
+        part_rr[(int64_t)blockIdx.x * Rs + threadIdx.x] = s;
+    }
+}
+
+__global__ void __launch_bounds__(kBlock) k_m_pupdate(int n, int R, int Rs, double* p, const double* __restrict__ z,
+                                                       float* p32, int first, const MultiState* st,
+                                                       const int* active) {
+    pdl_entry();
+    if (*active == 0) return;
+    const PairLayout P = pair_layout(Rs);
+    if (!P.in) return;
+    double beta[2];
+    bool on[2];
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+        on[j] = P.c + j < R && !st[P.c + j].done;
+        beta[j] = on[j] && !first ? st[P.c + j].beta : 0.0;
+    }
+    if (!on[0] && !on[1]) return;
+    for (int64_t i = (int64_t)blockIdx.x * P.rpb + P.rl; i < n; i += (int64_t)gridDim.x * P.rpb) {
+        const int64_t e = i * Rs + P.c;
+        double zv[2], pv[2];
+        load_vec<2>(z + e, zv);
+        load_vec<2>(p + e, pv);
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+            if (!on[j]) continue;
+            const double pi = first ? zv[j] : fma(beta[j], pv[j], zv[j]);
+            p[e + j] = pi;
+            if (p32) p32[e + j] = __double2float_rn(pi);
+        }
+    }
+}
+
+// --------------------------------------------------- kernels, batch of systems
+// A block per tile: rows [row0, row1) of one system.
+#define BATCH_TILE(T)                                       \
+    const int4 tile = (T)[blockIdx.x]; /* system, row0, row1 */ \
+    const int sys = tile.x, row0 = tile.y, row1 = tile.z;
+
+// tile partials of a.b and (c given) c.d; which: systems not done, or those
+// whose residual replacement is due
+__global__ void __launch_bounds__(kBlock) k_b_dots(const int4* __restrict__ tiles, const double* __restrict__ a,
+                                                    const double* __restrict__ b, const double* __restrict__ c,
+                                                    const double* __restrict__ d, double* part0, double* part1,
+                                                    int all, int due, const MultiState* st, const int* active) {
+    pdl_entry();
+    if (!all && *active == 0) return;
+    BATCH_TILE(tiles)
+    if (!all && (st[sys].done || (due && !st[sys].replace_now))) return;
+    __shared__ double sh[kWarpsPerBlock];
+    double s0 = 0.0, s1 = 0.0;
+    for (int i = row0 + threadIdx.x; i < row1; i += kBlock) {
+        s0 = fma(a[i], b[i], s0);
+        if (c) s1 = fma(c[i], d[i], s1);
+    }
+    block_partial(s0, sh, part0 + blockIdx.x);
+    if (c) block_partial(s1, sh, part1 + blockIdx.x);
+}
+
+template <typename X0>
+__global__ void __launch_bounds__(kBlock) k_b_update(const int4* __restrict__ tiles, double* x, double* r,
+                                                      const double* __restrict__ p, const double* __restrict__ q,
+                                                      const X0* __restrict__ invd, X0* x0, double* part_rr,
+                                                      const MultiState* st, const int* active) {
+    pdl_entry();
+    if (*active == 0) return;
+    BATCH_TILE(tiles)
+    if (st[sys].done) return;
+    __shared__ double sh[kWarpsPerBlock];
+    const double alpha = st[sys].alpha;
+    double rr = 0.0;
+    for (int i = row0 + threadIdx.x; i < row1; i += kBlock) {
+        x[i] = fma(alpha, p[i], x[i]);
+        const double ri = fma(-alpha, q[i], r[i]);
+        r[i] = ri;
+        if (x0) x0[i] = (X0)ri * invd[i];
+        rr = fma(ri, ri, rr);
+    }
+    block_partial(rr, sh, part_rr + blockIdx.x);
+}
+
+__global__ void __launch_bounds__(kBlock) k_b_pupdate(const int4* __restrict__ tiles, double* p,
+                                                       const double* __restrict__ z, float* p32, int first,
+                                                       const MultiState* st, const int* active) {
+    pdl_entry();
+    if (*active == 0) return;
+    BATCH_TILE(tiles)
+    if (st[sys].done) return;
+    const double beta = st[sys].beta;
+    for (int i = row0 + threadIdx.x; i < row1; i += kBlock) {
+        const double pi = first ? z[i] : fma(beta, p[i], z[i]);
+        p[i] = pi;
+        if (p32) p32[i] = __double2float_rn(pi);
+    }
+}
+
+// FP64 residual r = F - K x, x0 = r / d, of every system or (gate) of those
+// whose replacement is due; row groups without such a row are skipped.
+template <typename X0>
+__global__ void __launch_bounds__(kBlock) k_b_residual(int n, CsrM<double> mat, const double* __restrict__ x,
+                                                        const double* __restrict__ F, const X0* __restrict__ invd,
+                                                        double* r, X0* x0, const MultiState* st,
+                                                        const int32_t* __restrict__ seg, const unsigned* gate) {
+    pdl_entry();
+    if (gate && *gate == 0) return;
+    constexpr int RPW = 32;
+    ROWGROUP_PROLOGUE(double)
+    bool mine = owner;
+    if (gate) {
+        if (owner) {
+            const MultiState& m = st[seg[myrow]];
+            mine = !m.done && m.replace_now;
+        }
+        if (!__any_sync(FULL, mine)) return;
+    }
+    const double s = group_rows<RPW, double>(mat, x, row0, n, lane, tiles[wid]);
+    if (mine) {
+        const double ri = F[myrow] - s;
+        r[myrow] = ri;
+        if (x0) x0[myrow] = (X0)ri * invd[myrow];
     }
 }
 
 // ------------------------------------------------------------------ scalars
-// One block, one thread per system; *active = number of systems not done.
-__device__ void count_active(int S, const MultiState* st, int* active) {
+// Partial sums of one dot product per system: right-hand sides have nb block
+// partials of Rs columns each; a batch's system s has the tiles
+// [tile0[s], tile0[s + 1]).
+struct Parts {
+    int nb, Rs;
+    const int* tile0;
+};
+
+// tot[s] = sum of system s's partials, in a fixed order, for s < S (shared
+// memory; one block).  Right-hand sides: the block's threads split the block
+// partials of each column; batch: a warp per system.
+__device__ void sum_systems(const Parts& P, int S, const double* __restrict__ part, double* tot, double* sh) {
+    if (!P.tile0) {
+        const int per = blockDim.x / P.Rs, c = threadIdx.x % P.Rs, j = threadIdx.x / P.Rs;
+        double s = 0.0;
+        if (j < per) {
+#pragma unroll 8
+            for (int b = j; b < P.nb; b += per) s += part[(int64_t)b * P.Rs + c];
+        }
+        __syncthreads();
+        sh[threadIdx.x] = s;
+        // column c's `per` values, folded in half until one is left
+        for (int w = per; w > 1;) {
+            const int half = (w + 1) >> 1;
+            __syncthreads();
+            if (j + half < w) sh[threadIdx.x] += sh[threadIdx.x + half * P.Rs];
+            w = half;
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < S) tot[threadIdx.x] = sh[threadIdx.x];
+    } else {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        __syncthreads();
+        for (int s = wid; s < S; s += nw) {
+            double t = 0.0;
+            for (int k = P.tile0[s] + lane; k < P.tile0[s + 1]; k += 32) t += part[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+            if (lane == 0) tot[s] = t;
+        }
+    }
+    __syncthreads();
+}
+
+constexpr int kScalThreads = 1024;
+#define SCAL_SHARED                      \
+    __shared__ double sh[kScalThreads]; \
+    __shared__ double t0[kScalThreads];
+
+// *active = number of systems not done (0 as well once the single-system
+// state, which the batch's V-cycle kernels read, says stop).
+__device__ void count_active(int S, const MultiState* st, int* active, SolveState* single) {
     __shared__ int cnt;
+    __syncthreads();
     if (threadIdx.x == 0) cnt = 0;
     __syncthreads();
     for (int s = threadIdx.x; s < S; s += blockDim.x)
         if (!st[s].done) atomicAdd(&cnt, 1);
     __syncthreads();
-    if (threadIdx.x == 0) *active = cnt;
+    if (threadIdx.x == 0) {
+        const int a = single->done ? 0 : cnt;
+        *active = a;
+        if (a == 0) single->done = 1;
+    }
 }
 
-__global__ void k_m_scal_init(int S, const double* dots, double rtol, int itmax, int repl, MultiState* st,
-                              int* active, int* itmax_out) {
+// all systems' squared norms of the start residual and of F
+__global__ void __launch_bounds__(kScalThreads) k_m_scal_init(Parts P, int S, const double* part_rr,
+                                                               const double* part_ff, double rtol, int itmax,
+                                                               int repl, MultiState* st, int* active, int* itmax_out,
+                                                               unsigned* due, SolveState* single) {
+    pdl_entry();
+    SCAL_SHARED
+    __shared__ double t1[kScalThreads];
+    sum_systems(P, S, part_rr, t0, sh);
+    sum_systems(P, S, part_ff, t1, sh);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         MultiState& m = st[s];
-        const double nF = sqrt(dots[s * D_COUNT + D_FF]), nr = sqrt(dots[s * D_COUNT + D_RR]);
+        const double nF = sqrt(t1[s]), nr = sqrt(t0[s]);
         m.nF = nF;
         m.tol = rtol * nF;
         m.nr = nr;
@@ -304,17 +829,27 @@ __global__ void k_m_scal_init(int S, const double* dots, double rtol, int itmax,
     if (threadIdx.x == 0) {
         itmax_out[0] = itmax;
         itmax_out[1] = repl;
+        *due = 0;
+        single->done = 0;
+        single->status = AMG_OK;
     }
-    count_active(S, st, active);
+    count_active(S, st, active, single);
 }
 
-__global__ void k_m_scal_alpha(int S, const double* dots, int flexible, MultiState* st, int* active) {
+__global__ void __launch_bounds__(kScalThreads) k_m_scal_alpha(Parts P, int S, const double* part_pq,
+                                                                const double* part_pr, int flexible, MultiState* st,
+                                                                int* active, SolveState* single) {
+    pdl_entry();
     if (*active == 0) return;
+    SCAL_SHARED
+    __shared__ double t1[kScalThreads];
+    sum_systems(P, S, part_pq, t0, sh);
+    if (flexible) sum_systems(P, S, part_pr, t1, sh);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         MultiState& m = st[s];
         if (m.done) continue;
-        const double pq = dots[s * D_COUNT + D_PQ];
-        const double num = flexible ? dots[s * D_COUNT + D_PR] : m.rho;
+        const double pq = t0[s];
+        const double num = flexible ? t1[s] : m.rho;
         m.pq = pq;
         if (!(pq > 0.0)) {
             m.status = (isnan(pq) || isnan(num)) ? AMG_ERR_NAN : AMG_ERR_BREAKDOWN;
@@ -323,16 +858,25 @@ __global__ void k_m_scal_alpha(int S, const double* dots, int flexible, MultiSta
             m.alpha = num / pq;
         }
     }
-    count_active(S, st, active);
+    count_active(S, st, active, single);
 }
 
-__global__ void k_m_scal_conv(int S, const double* dots, int mixed, const int* params, MultiState* st, int* active) {
+// *due: the right-hand sides (bit s) whose FP64 residual replacement is due;
+// nonzero for a batch when any system's is.
+__global__ void __launch_bounds__(kScalThreads) k_m_scal_conv(Parts P, int S, const double* part_rr, int mixed,
+                                                               const int* params, MultiState* st, int* active,
+                                                               unsigned* due, SolveState* single) {
+    pdl_entry();
     if (*active == 0) return;
+    SCAL_SHARED
+    __shared__ unsigned mask;
+    if (threadIdx.x == 0) mask = 0;
+    sum_systems(P, S, part_rr, t0, sh);
     const int itmax = params[0], repl = params[1];
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         MultiState& m = st[s];
         if (m.done) continue;
-        const double nr = sqrt(dots[s * D_COUNT + D_RR]);
+        const double nr = sqrt(t0[s]);
         const int it = m.iters + 1;
         m.iters = it;
         m.nr = nr;
@@ -341,6 +885,7 @@ __global__ void k_m_scal_conv(int S, const double* dots, int mixed, const int* p
             m.done = 1;
         } else if (mixed && (nr <= m.tol || it >= itmax || (repl > 0 && it % repl == 0))) {
             m.replace_now = 1;
+            atomicOr(&mask, 1u << (s & 31));
         } else if (nr <= m.tol) {
             m.done = 1;
         } else if (it >= itmax) {
@@ -348,16 +893,23 @@ __global__ void k_m_scal_conv(int S, const double* dots, int mixed, const int* p
             m.done = 1;
         }
     }
-    count_active(S, st, active);
+    __syncthreads();
+    if (threadIdx.x == 0) *due = mask;
+    count_active(S, st, active, single);
 }
 
-__global__ void k_m_scal_replaced(int S, const double* dots, const int* params, MultiState* st, int* active) {
-    if (*active == 0) return;
+__global__ void __launch_bounds__(kScalThreads) k_m_scal_replaced(Parts P, int S, const double* part_rr,
+                                                                   const int* params, MultiState* st, int* active,
+                                                                   unsigned* due, SolveState* single) {
+    pdl_entry();
+    if (*active == 0 || *due == 0) return;
+    SCAL_SHARED
+    sum_systems(P, S, part_rr, t0, sh);
     const int itmax = params[0];
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         MultiState& m = st[s];
         if (m.done || !m.replace_now) continue;
-        const double nr = sqrt(dots[s * D_COUNT + D_RR2]);
+        const double nr = sqrt(t0[s]);
         m.nr = nr;
         m.replace_now = 0;
         if (isnan(nr) || isinf(nr)) {
@@ -370,40 +922,63 @@ __global__ void k_m_scal_replaced(int S, const double* dots, const int* params, 
             m.done = 1;
         }
     }
-    count_active(S, st, active);
+    if (threadIdx.x == 0) *due = 0;
+    count_active(S, st, active, single);
 }
 
-__global__ void k_m_scal_beta(int S, const double* dots, int flexible, int first, MultiState* st, int* active) {
+__global__ void __launch_bounds__(kScalThreads) k_m_scal_beta(Parts P, int S, const double* part_rz,
+                                                               const double* part_zq, int flexible, int first,
+                                                               MultiState* st, int* active, SolveState* single) {
+    pdl_entry();
     if (*active == 0) return;
+    SCAL_SHARED
+    __shared__ double t1[kScalThreads];
+    const bool flex = flexible && !first;
+    sum_systems(P, S, part_rz, t0, sh);
+    if (flex) sum_systems(P, S, part_zq, t1, sh);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         MultiState& m = st[s];
         if (m.done) continue;
-        const double rz = dots[s * D_COUNT + D_RZ];
-        const double zq = dots[s * D_COUNT + D_ZQ];
-        if (isnan(rz) || (flexible && !first && isnan(zq))) {
+        const double rz = t0[s];
+        if (isnan(rz) || (flex && isnan(t1[s]))) {
             m.status = AMG_ERR_NAN;
             m.done = 1;
             continue;
         }
-        m.beta = first ? 0.0 : (flexible ? -zq / m.pq : rz / m.rho);
+        m.beta = first ? 0.0 : (flexible ? -t1[s] / m.pq : rz / m.rho);
         m.rho = rz;
     }
-    count_active(S, st, active);
+    count_active(S, st, active, single);
 }
 
-// [N][R] <-> column-major (leading dimension ld) copies
-__global__ void k_interleave(int n, int R, int64_t ld, const double* __restrict__ src, double* dst) {
+// dots[2 s], dots[2 s + 1] = the systems' sums (the final residual norms)
+__global__ void __launch_bounds__(kScalThreads) k_m_totals(Parts P, int S, const double* part0, const double* part1,
+                                                            double* dots) {
+    pdl_entry();
+    SCAL_SHARED
+    __shared__ double t1[kScalThreads];
+    sum_systems(P, S, part0, t0, sh);
+    sum_systems(P, S, part1, t1, sh);
+    for (int s = threadIdx.x; s < S; s += blockDim.x) {
+        dots[2 * s] = t0[s];
+        dots[2 * s + 1] = t1[s];
+    }
+}
+
+// [N][Rs] <-> column-major (leading dimension ld) copies; the padding
+// columns become zero
+__global__ void k_interleave(int n, int R, int Rs, int64_t ld, const double* __restrict__ src, double* dst) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= (int64_t)n * R) return;
-    const int i = (int)(g / R), c = (int)(g % R);
-    dst[g] = src[(int64_t)c * ld + i];
+    if (g >= (int64_t)n * Rs) return;
+    const int i = (int)(g / Rs), c = (int)(g % Rs);
+    dst[g] = c < R ? src[(int64_t)c * ld + i] : 0.0;
 }
 
-__global__ void k_deinterleave(int n, int R, int64_t ld, const double* __restrict__ src, double* dst) {
+__global__ void k_deinterleave(int n, int R, int Rs, int64_t ld, const double* __restrict__ src, double* dst) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (g >= (int64_t)n * R) return;
     const int i = (int)(g % n), c = (int)(g / n);
-    dst[(int64_t)c * ld + i] = src[(int64_t)i * R + c];
+    dst[(int64_t)c * ld + i] = src[(int64_t)i * Rs + c];
 }
 
 // ----------------------------------------------------------------- host side
@@ -438,169 +1013,308 @@ struct MView<float> {
 template <typename T>
 using vt = std::remove_cv_t<std::remove_pointer_t<T>>;
 
+template <typename V>
+MatM<V> mat_of(const Level& L, const V* v) {
+    return MatM<V>{L.A.rowptr, L.A.col, v, L.run_ptr, L.run_len, L.run_start};
+}
+
+enum { M_A = 0, M_B, M_SLOTS };  // partial-sum slots (two dot products at a time)
+double* mslot(MultiWork& w, int k) { return w.part + (int64_t)k * w.part_stride; }
+
+// lanes per entry: 16 bytes of the Rs columns each, a power of two
+template <typename A>
+int lanes_per_entry(int Rs) {
+    const int q = Rs / kVec<A>;
+    int p = 1;
+    while (p < q) p <<= 1;
+    return p;
+}
+
+// Rows of a block that share one epilogue: all copies of a column where the
+// level has rows enough to fill the GPU's warps that way, else one.
+template <typename A>
+int rows_together(amg_hierarchy* h, int n, int Rs) {
+    const int t = 32 / (kVec<A> * lanes_per_entry<A>(Rs));
+    return (int64_t)n >= (int64_t)h->num_sms * 16 * t ? t : 1;
+}
+
+// blocks of the SpMM kernels: two per SM (the partial sums of a dot product
+// are one per block, and their sum is FP64 work of one SM)
+int spmm_blocks(amg_hierarchy* h, int n) {
+    const int64_t b = ((int64_t)n + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    const int64_t cap = (int64_t)h->num_sms * 2;
+    return (int)(b < cap ? b : cap);
+}
+int coarse_blocks(amg_hierarchy* h) {
+    const int cap = h->num_sms * 2;
+    return h->ndense < cap ? h->ndense : cap;
+}
+
+// blocks of the vector kernels of R right-hand sides
+int pair_blocks(amg_hierarchy* h, int n, int Rs) {
+    const int rpb = kBlock / (Rs / 2);
+    const int64_t b = ((int64_t)n + rpb - 1) / rpb;
+    const int64_t cap = (int64_t)h->num_sms * 2;
+    return (int)(b < cap ? b : cap);
+}
+
+// fn(true) where the finest level has run-encoded columns and the products
+// are FP32, else fn(false): in FP64 the pass is bound by the FP64 pipe, and
+// taking four rows at once only costs warps in flight (3-D p = 3 n = 24, 16
+// right-hand sides: 135 ms a solve against 76 ms row by row).
+template <typename A, typename Fn>
+void with_runs(const Level& L, Fn&& fn) {
+    if constexpr (std::is_same_v<A, float>) {
+        if (L.run_ptr) {
+            fn(std::true_type{});
+            return;
+        }
+    }
+    fn(std::false_type{});
+}
+
 template <typename A>
 cudaError_t m_vcycle(amg_hierarchy* h, cudaStream_t s) {
     using Vw = MView<A>;
     MultiWork& w = *h->mw;
-    const int L = h->nlev, R = w.R, Rp = w.Rp, flex = h->o.flexible;
+    const int L = h->nlev, Rs = w.Rs, lp = lanes_per_entry<A>(Rs), flex = h->o.flexible;
     const int* act = w.active;
     if (L == 1) {
-        k_m_coarse<double, A><<<AMG_GRID(elem_blocks((int64_t)h->ndense * R)), 256, 0, s>>>(
-            h->ndense, R, h->Ainv, w.r, nullptr, nullptr, nullptr, nullptr, w.z, w.q, w.pa, w.pb, flex, act);
+        launch_pdl(k_m_coarse<double, A>, coarse_blocks(h), 32, 0, s, h->ndense, Rs,
+                   lanes_per_entry<double>(Rs), h->Ainv, w.r, nullptr, nullptr, nullptr, nullptr, w.z, w.q,
+                   mslot(w, M_A), mslot(w, M_B), flex, act);
         return cudaGetLastError();
     }
     for (int l = 0; l < L - 1; l++) {
         Level& F = h->lev[l];
         Level& C = h->lev[l + 1];
-        const int n = F.A.n;
-        const int nb = elem_blocks((int64_t)n * Rp);
+        const int n = F.A.n, nb = spmm_blocks(h, n), T = rows_together<A>(h, n, Rs);
         Vw::vals(F, l, [&](auto vp) {
             using V = vt<decltype(vp)>;
             if (l == 0)
-                k_m_resid<A, V, double><<<AMG_GRID(nb), 256, 0, s>>>(n, R, Rp, F.A.rowptr, F.A.col, vp, w.r,
-                                                                     Vw::x(w, 0), Vw::t(w, 0), act);
+                with_runs<A>(F, [&](auto rn) {
+                    launch_pdl(k_m_resid<decltype(rn)::value, A, V, double>, nb, kBlock, 0, s, n, Rs, lp, T, mat_of(F, vp), w.r,
+                               Vw::x(w, 0), Vw::t(w, 0), act);
+                });
             else
-                k_m_resid<A, V, A><<<AMG_GRID(nb), 256, 0, s>>>(n, R, Rp, F.A.rowptr, F.A.col, vp, Vw::f(w, l),
-                                                                Vw::x(w, l), Vw::t(w, l), act);
+                launch_pdl(k_m_resid<false, A, V, A>, nb, kBlock, 0, s, n, Rs, lp, T, mat_of(F, vp), Vw::f(w, l),
+                           Vw::x(w, l), Vw::t(w, l), act);
         });
         const bool coarsest = (l + 1 == L - 1);
-        k_m_restrict<A><<<AMG_GRID(elem_blocks((int64_t)C.A.n * R)), 256, 0, s>>>(
-            C.A.n, R, F.mem_ptr, F.mem_idx, F.pval, Vw::t(w, l), Vw::f(w, l + 1), coarsest ? nullptr : Vw::x(w, l + 1),
-            Vw::invd(C), act);
+        launch_pdl(k_m_restrict<A>, elem_blocks((int64_t)C.A.n * Rs), 256, 0, s, C.A.n, Rs, F.mem_ptr, F.mem_idx,
+                   F.pval, Vw::t(w, l), Vw::f(w, l + 1), coarsest ? nullptr : Vw::x(w, l + 1), Vw::invd(C), act);
     }
     {
         Level& F = h->lev[L - 2];
         Level& C = h->lev[L - 1];
-        k_m_coarse<A, A><<<AMG_GRID(elem_blocks((int64_t)C.A.n * R)), 256, 0, s>>>(
-            C.A.n, R, h->Ainv, Vw::f(w, L - 1), F.mem_ptr, F.mem_idx, F.pval, Vw::x(w, L - 2), nullptr, nullptr,
-            nullptr, nullptr, 0, act);
+        launch_pdl(k_m_coarse<A, A>, coarse_blocks(h), 32, 0, s, C.A.n, Rs, lanes_per_entry<double>(Rs),
+                   h->Ainv, Vw::f(w, L - 1), F.mem_ptr, F.mem_idx, F.pval, Vw::x(w, L - 2), nullptr, nullptr, nullptr,
+                   nullptr, 0, act);
     }
     for (int l = L - 2; l >= 0; l--) {
         Level& F = h->lev[l];
-        const int n = F.A.n;
-        const int nb = elem_blocks((int64_t)n * Rp);
+        const int n = F.A.n, nb = spmm_blocks(h, n), T = rows_together<A>(h, n, Rs);
         Vw::vals(F, l, [&](auto vp) {
             using V = vt<decltype(vp)>;
             if (l == 0) {
-                k_m_up0<A, V><<<AMG_GRID(nb), 256, 0, s>>>(n, R, Rp, F.A.rowptr, F.A.col, vp, w.r, Vw::x(w, 0),
-                                                           Vw::invd(F), w.z, w.q, w.pa, w.pb, flex, act);
+                with_runs<A>(F, [&](auto rn) {
+                    launch_pdl(k_m_up0<decltype(rn)::value, A, V>, nb, kBlock, 0, s, n, Rs, lp, T, mat_of(F, vp), w.r, Vw::x(w, 0),
+                               Vw::invd(F), w.z, w.q, mslot(w, M_A), mslot(w, M_B), flex, act);
+                });
             } else {
                 Level& G = h->lev[l - 1];
-                k_m_up<A, V><<<AMG_GRID(nb), 256, 0, s>>>(n, R, Rp, F.A.rowptr, F.A.col, vp, Vw::f(w, l),
-                                                          Vw::x(w, l), Vw::invd(F), G.mem_ptr, G.mem_idx, G.pval,
-                                                          Vw::x(w, l - 1), act);
+                launch_pdl(k_m_up<A, V>, nb, kBlock, 0, s, n, Rs, lp, T, mat_of(F, vp), Vw::f(w, l),
+                           Vw::x(w, l), Vw::invd(F), G.mem_ptr, G.mem_idx, G.pval, Vw::x(w, l - 1), act);
             }
         });
     }
     return cudaGetLastError();
 }
 
-cudaError_t m_vcycle_any(amg_hierarchy* h, cudaStream_t s) {
-    return h->mixed ? m_vcycle<float>(h, s) : m_vcycle<double>(h, s);
+// Block partials of the kernels: right-hand sides, from the SpMM kernels or
+// (vec) from the vector kernels; a batch, from the tiles.
+Parts spmm_parts(amg_hierarchy* h) { return Parts{spmm_blocks(h, h->lev[0].A.n), h->mw->Rs, nullptr}; }
+Parts pair_parts(amg_hierarchy* h) {
+    return Parts{pair_blocks(h, h->lev[0].A.n, h->mw->Rs), h->mw->Rs, nullptr};
 }
+Parts tile_parts(amg_hierarchy* h) { return Parts{0, 0, h->mw->tile0}; }
 
-cudaError_t m_residual(amg_hierarchy* h, double* r, bool x0, bool ff, const MultiState* gate, cudaStream_t s) {
+// z = B r; r.z and z.q into the two slots; returns where their partials are
+cudaError_t any_vcycle(amg_hierarchy* h, Parts* P, cudaStream_t s) {
     MultiWork& w = *h->mw;
-    Level& L0 = h->lev[0];
-    const int n = L0.A.n;
-    const int nb = elem_blocks((int64_t)n * w.Rp);
-    const bool want = x0 && h->nlev > 1;
-    if (h->mixed)
-        k_m_residual<float><<<AMG_GRID(nb), 256, 0, s>>>(n, w.R, w.Rp, L0.A.rowptr, L0.A.col, L0.A.val, w.x, w.F,
-                                                         L0.invd32, r, want ? static_cast<float*>(w.lx[0]) : nullptr,
-                                                         w.pa, ff ? w.pb : nullptr, gate, w.seg);
-    else
-        k_m_residual<double><<<AMG_GRID(nb), 256, 0, s>>>(n, w.R, w.Rp, L0.A.rowptr, L0.A.col, L0.A.val, w.x, w.F,
-                                                          L0.invd, r, want ? static_cast<double*>(w.lx[0]) : nullptr,
-                                                          w.pa, ff ? w.pb : nullptr, gate, w.seg);
+    const int flex = h->o.flexible;
+    if (!w.tiles) {
+        AMG_TRY(h->mixed ? m_vcycle<float>(h, s) : m_vcycle<double>(h, s));
+        *P = h->nlev > 1 ? spmm_parts(h) : Parts{coarse_blocks(h), w.Rs, nullptr};
+        return cudaSuccess;
+    }
+    AMG_TRY(enqueue_vcycle_rows(h, s));
+    launch_pdl(k_b_dots, w.ntiles, kBlock, 0, s, w.tiles, w.r, w.z, flex ? w.z : nullptr, w.q, mslot(w, M_A),
+               mslot(w, M_B), 0, 0, w.st, w.active);
+    *P = tile_parts(h);
     return cudaGetLastError();
 }
 
-void m_sum(amg_hierarchy* h, const double* pa, int sa, const double* pb, int sb, const int* act, cudaStream_t s) {
+// r = F - K x, x0 = r / d; r.r (slot A) and, with ff, F.F (slot B).  due:
+// only the systems whose replacement is due.
+cudaError_t any_residual(amg_hierarchy* h, double* r, bool x0, bool ff, bool due, Parts* P, cudaStream_t s) {
     MultiWork& w = *h->mw;
-    k_m_sys_sum<<<AMG_GRID(w.S), 256, 0, s>>>(h->lev[0].A.n, w.R, w.segoff, pa, sa, pb, sb, w.dots, act);
+    Level& L0 = h->lev[0];
+    const int n = L0.A.n;
+    const bool want = x0 && h->nlev > 1;
+    const unsigned* gate = due ? w.due : nullptr;
+    if (!w.tiles) {
+        const int nb = spmm_blocks(h, n), lp = lanes_per_entry<double>(w.Rs);
+        const int T = rows_together<double>(h, n, w.Rs);
+        double* pff = ff ? mslot(w, M_B) : nullptr;
+        const auto mat = mat_of(L0, static_cast<const double*>(L0.A.val));
+        if (h->mixed)
+            launch_pdl(k_m_residual<float>, nb, kBlock, 0, s, n, w.Rs, lp, T, mat, w.x, w.F, L0.invd32, r,
+                       want ? static_cast<float*>(w.lx[0]) : nullptr, mslot(w, M_A), pff, gate);
+        else
+            launch_pdl(k_m_residual<double>, nb, kBlock, 0, s, n, w.Rs, lp, T, mat, w.x, w.F, L0.invd, r,
+                       want ? static_cast<double*>(w.lx[0]) : nullptr, mslot(w, M_A), pff, gate);
+        *P = spmm_parts(h);
+        return cudaGetLastError();
+    }
+    // the FP64 matrix (also in mixed precision), a row per lane
+    const CsrM<double> mat{L0.A.rowptr, L0.A.col, L0.A.val};
+    const int nb = row_blocks(n, 32);
+    if (h->mixed)
+        launch_pdl(k_b_residual<float>, nb, kBlock, 0, s, n, mat, w.x, w.F, L0.invd32, r, want ? L0.x32 : nullptr,
+                   w.st, w.seg, gate);
+    else
+        launch_pdl(k_b_residual<double>, nb, kBlock, 0, s, n, mat, w.x, w.F, L0.invd, r, want ? L0.x : nullptr, w.st,
+                   w.seg, gate);
+    launch_pdl(k_b_dots, w.ntiles, kBlock, 0, s, w.tiles, r, r, ff ? w.F : nullptr, w.F, mslot(w, M_A),
+               mslot(w, M_B), due ? 0 : 1, due ? 1 : 0, w.st, w.active);
+    *P = tile_parts(h);
+    return cudaGetLastError();
 }
 
-void m_pupdate(amg_hierarchy* h, int first, cudaStream_t s) {
+void any_pupdate(amg_hierarchy* h, int first, cudaStream_t s) {
     MultiWork& w = *h->mw;
-    const int64_t cnt = (int64_t)h->lev[0].A.n * w.R;
-    k_m_pupdate<<<AMG_GRID(elem_blocks(cnt)), 256, 0, s>>>(h->lev[0].A.n, w.R, w.p, w.z, h->mixed ? w.p32 : nullptr,
-                                                           first, w.st, w.seg, w.active);
+    float* p32 = h->mixed ? w.p32 : nullptr;
+    if (w.tiles)
+        launch_pdl(k_b_pupdate, w.ntiles, kBlock, 0, s, w.tiles, w.p, w.z, p32, first, w.st, w.active);
+    else
+        launch_pdl(k_m_pupdate, pair_blocks(h, h->lev[0].A.n, w.Rs), kBlock, 0, s, h->lev[0].A.n, w.R, w.Rs, w.p,
+                   w.z, p32, first, w.st, w.active);
+}
+
+// q = K p with p.q (slot A) and, flexible, p.r (slot B)
+cudaError_t any_spmv_pq(amg_hierarchy* h, Parts* P, cudaStream_t s) {
+    MultiWork& w = *h->mw;
+    Level& L0 = h->lev[0];
+    const int n = L0.A.n, flex = h->o.flexible;
+    if (w.tiles) {
+        AMG_TRY(launch_rowgroup_pq(h, s, true));
+        launch_pdl(k_b_dots, w.ntiles, kBlock, 0, s, w.tiles, w.p, w.q, flex ? w.p : nullptr, w.r, mslot(w, M_A),
+                   mslot(w, M_B), 0, 0, w.st, w.active);
+        *P = tile_parts(h);
+        return cudaGetLastError();
+    }
+    const int nb = spmm_blocks(h, n);
+    if (h->mixed)
+        with_runs<float>(L0, [&](auto rn) {
+            launch_pdl(k_m_spmv_pq<decltype(rn)::value, float, float>, nb, kBlock, 0, s, n, w.Rs,
+                       lanes_per_entry<float>(w.Rs), rows_together<float>(h, n, w.Rs),
+                       mat_of(L0, static_cast<const float*>(L0.val32)), w.p32, w.p, w.r, w.q, mslot(w, M_A),
+                       mslot(w, M_B), flex, w.active);
+        });
+    else
+        launch_pdl(k_m_spmv_pq<false, double, double>, nb, kBlock, 0, s, n, w.Rs, lanes_per_entry<double>(w.Rs),
+                   rows_together<double>(h, n, w.Rs), mat_of(L0, static_cast<const double*>(L0.A.val)), w.p, w.p,
+                   w.r, w.q, mslot(w, M_A), mslot(w, M_B), flex, w.active);
+    *P = spmm_parts(h);
+    return cudaGetLastError();
+}
+
+// x += alpha p, r -= alpha q, x0 = r / d, r.r (slot A)
+cudaError_t any_update(amg_hierarchy* h, Parts* P, cudaStream_t s) {
+    MultiWork& w = *h->mw;
+    Level& L0 = h->lev[0];
+    const bool x0 = h->nlev > 1;
+    auto launch = [&](auto* invd, auto* xb, auto* xm) {
+        using X0 = std::remove_pointer_t<decltype(xm)>;
+        if (w.tiles)
+            launch_pdl(k_b_update<X0>, w.ntiles, kBlock, 0, s, w.tiles, w.x, w.r, w.p, w.q, invd,
+                       x0 ? xb : nullptr, mslot(w, M_A), w.st, w.active);
+        else
+            launch_pdl(k_m_update<X0>, pair_blocks(h, L0.A.n, w.Rs), kBlock, 0, s, L0.A.n, w.R, w.Rs, w.x, w.r, w.p,
+                       w.q, invd, x0 ? xm : nullptr, mslot(w, M_A), w.st, w.active);
+    };
+    if (h->mixed) launch(static_cast<const float*>(L0.invd32), L0.x32, static_cast<float*>(w.lx[0]));
+    else launch(static_cast<const double*>(L0.invd), L0.x, static_cast<double*>(w.lx[0]));
+    *P = w.tiles ? tile_parts(h) : pair_parts(h);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
+// Doubles of one partial-sum slot: the block partials of R interleaved
+// right-hand sides, or one per tile.
+size_t multi_part_stride(amg_hierarchy* h, int Rs, int ntiles) {
+    if (ntiles > 0) return (size_t)ntiles;
+    const size_t a = (size_t)spmm_blocks(h, h->lev[0].A.n), b = (size_t)pair_blocks(h, h->lev[0].A.n, Rs);
+    const size_t c = (size_t)coarse_blocks(h);  // a single-level hierarchy
+    return std::max(std::max(a, b), c) * Rs;
+}
+int multi_part_slots() { return M_SLOTS; }
+
 cudaError_t enqueue_multi_start(amg_hierarchy* h, cudaStream_t s) {
     MultiWork& w = *h->mw;
-    AMG_TRY(m_residual(h, w.r, true, true, nullptr, s));
-    m_sum(h, w.pa, D_RR, w.pb, D_FF, nullptr, s);
-    k_m_scal_init<<<AMG_GRID(1), 1024, 0, s>>>(w.S, w.dots, h->rtol, h->itmax,
-                                               h->mixed ? h->o.resid_replace_every : 0, w.st, w.active, w.params);
+    Parts P;
+    AMG_TRY(any_residual(h, w.r, true, true, false, &P, s));
+    launch_pdl(k_m_scal_init, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), h->rtol, h->itmax,
+               h->mixed ? h->o.resid_replace_every : 0, w.st, w.active, w.params, w.due, h->st);
     AMG_TRY(cudaGetLastError());
-    AMG_TRY(m_vcycle_any(h, s));
-    m_sum(h, w.pa, D_RZ, h->o.flexible ? w.pb : nullptr, D_ZQ, w.active, s);
-    k_m_scal_beta<<<AMG_GRID(1), 1024, 0, s>>>(w.S, w.dots, h->o.flexible, 1, w.st, w.active);
-    m_pupdate(h, 1, s);
+    AMG_TRY(any_vcycle(h, &P, s));
+    launch_pdl(k_m_scal_beta, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), h->o.flexible, 1, w.st,
+               w.active, h->st);
+    any_pupdate(h, 1, s);
     return cudaGetLastError();
 }
 
 cudaError_t enqueue_multi_iteration(amg_hierarchy* h, cudaStream_t s) {
     MultiWork& w = *h->mw;
-    Level& L0 = h->lev[0];
-    const int n = L0.A.n, R = w.R, Rp = w.Rp, flex = h->o.flexible;
-    const int nb = elem_blocks((int64_t)n * Rp);
-    if (h->mixed)
-        k_m_spmv_pq<float, float, float><<<AMG_GRID(nb), 256, 0, s>>>(n, R, Rp, L0.A.rowptr, L0.A.col, L0.val32,
-                                                                      w.p32, w.p, w.r, w.q, w.pa, w.pb, flex, w.st,
-                                                                      w.seg, w.active);
-    else
-        k_m_spmv_pq<double, double, double><<<AMG_GRID(nb), 256, 0, s>>>(n, R, Rp, L0.A.rowptr, L0.A.col, L0.A.val,
-                                                                         w.p, w.p, w.r, w.q, w.pa, w.pb, flex, w.st,
-                                                                         w.seg, w.active);
-    m_sum(h, w.pa, D_PQ, flex ? w.pb : nullptr, D_PR, w.active, s);
-    k_m_scal_alpha<<<AMG_GRID(1), 1024, 0, s>>>(w.S, w.dots, flex, w.st, w.active);
-    const int64_t cnt = (int64_t)n * R;
-    const bool x0 = h->nlev > 1;
-    if (h->mixed)
-        k_m_update<float><<<AMG_GRID(elem_blocks(cnt)), 256, 0, s>>>(
-            n, R, w.x, w.r, w.p, w.q, L0.invd32, x0 ? static_cast<float*>(w.lx[0]) : nullptr, w.pa, w.st, w.seg,
-            w.active);
-    else
-        k_m_update<double><<<AMG_GRID(elem_blocks(cnt)), 256, 0, s>>>(
-            n, R, w.x, w.r, w.p, w.q, L0.invd, x0 ? static_cast<double*>(w.lx[0]) : nullptr, w.pa, w.st, w.seg,
-            w.active);
-    m_sum(h, w.pa, D_RR, nullptr, 0, w.active, s);
-    k_m_scal_conv<<<AMG_GRID(1), 1024, 0, s>>>(w.S, w.dots, h->mixed, w.params, w.st, w.active);
-    if (h->mixed) {
-        AMG_TRY(m_residual(h, w.r, true, false, w.st, s));
-        m_sum(h, w.pa, D_RR2, nullptr, 0, w.active, s);
-        k_m_scal_replaced<<<AMG_GRID(1), 1024, 0, s>>>(w.S, w.dots, w.params, w.st, w.active);
+    const int flex = h->o.flexible;
+    Parts P;
+    AMG_TRY(any_spmv_pq(h, &P, s));
+    launch_pdl(k_m_scal_alpha, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), flex, w.st, w.active,
+               h->st);
+    AMG_TRY(any_update(h, &P, s));
+    launch_pdl(k_m_scal_conv, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), h->mixed, w.params, w.st, w.active,
+               w.due, h->st);
+    if (h->mixed) {  // FP64 true-residual replacement, when due
+        AMG_TRY(any_residual(h, w.r, true, false, true, &P, s));
+        launch_pdl(k_m_scal_replaced, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), w.params, w.st, w.active, w.due,
+                   h->st);
     }
     AMG_TRY(cudaGetLastError());
-    AMG_TRY(m_vcycle_any(h, s));
-    m_sum(h, w.pa, D_RZ, flex ? w.pb : nullptr, D_ZQ, w.active, s);
-    k_m_scal_beta<<<AMG_GRID(1), 1024, 0, s>>>(w.S, w.dots, flex, 0, w.st, w.active);
-    m_pupdate(h, 0, s);
+    AMG_TRY(any_vcycle(h, &P, s));
+    launch_pdl(k_m_scal_beta, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), flex, 0, w.st, w.active,
+               h->st);
+    any_pupdate(h, 0, s);
     return cudaGetLastError();
 }
 
-// ||F_s - K x_s|| and ||F_s|| per system into dots[s][RR], dots[s][FF].
+// ||F_s - K x_s||^2 and ||F_s||^2 per system into dots[2 s], dots[2 s + 1].
 cudaError_t enqueue_multi_final(amg_hierarchy* h, cudaStream_t s) {
     MultiWork& w = *h->mw;
-    AMG_TRY(m_residual(h, w.q, false, true, nullptr, s));
-    m_sum(h, w.pa, D_RR, w.pb, D_FF, nullptr, s);
+    Parts P;
+    AMG_TRY(any_residual(h, w.q, false, true, false, &P, s));
+    launch_pdl(k_m_totals, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), w.dots);
     return cudaGetLastError();
 }
 
-int multi_dot_stride() { return D_COUNT; }
-
-cudaError_t launch_interleave(int n, int R, int64_t ld, const double* src, double* dst, cudaStream_t s) {
-    k_interleave<<<AMG_GRID(elem_blocks((int64_t)n * R)), 256, 0, s>>>(n, R, ld, src, dst);
+cudaError_t launch_interleave(int n, int R, int Rs, int64_t ld, const double* src, double* dst, cudaStream_t s) {
+    k_interleave<<<AMG_GRID(elem_blocks((int64_t)n * Rs)), 256, 0, s>>>(n, R, Rs, ld, src, dst);
     return cudaGetLastError();
 }
 
-cudaError_t launch_deinterleave(int n, int R, int64_t ld, const double* src, double* dst, cudaStream_t s) {
-    k_deinterleave<<<AMG_GRID(elem_blocks((int64_t)n * R)), 256, 0, s>>>(n, R, ld, src, dst);
+cudaError_t launch_deinterleave(int n, int R, int Rs, int64_t ld, const double* src, double* dst, cudaStream_t s) {
+    k_deinterleave<<<AMG_GRID(elem_blocks((int64_t)n * R)), 256, 0, s>>>(n, R, Rs, ld, src, dst);
     return cudaGetLastError();
 }
 
