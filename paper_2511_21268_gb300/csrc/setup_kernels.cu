@@ -1332,7 +1332,209 @@ __global__ void k_dense_from_csr(int n, const int64_t* __restrict__ rp, const in
     }
 }
 
-// Right-looking Cholesky D = L L^T in place (lower triangle, one block).
+// Correctly rounded square root (IEEE binary64, round to nearest even) of a
+// positive normal a of moderate exponent in eight FP64 operations, in the
+// manner of div_rn (amg_internal.cuh): the SFU's FP32 reciprocal root of the
+// leading bits, one coupled Newton step for g ~ sqrt(a) and h ~ 1 / (2
+// sqrt(a)) (Goldschmidt; error below 2^-42), a correction g += (a - g^2) h,
+// and an exact acceptance test: the remainder e = a - s^2 of a faithful root
+// s is a double (Boldo and Daumas 2003, as for div_rn), and s = RN(sqrt(a))
+// if |e| < s ulp(s) (no square root of a double lies half-way between two
+// doubles; e and s ulp(s) are multiples of ulp(s)^2, so the square of the
+// half-gap cannot decide).  Roots at a power of two, where the gap below is
+// half as wide, and operands outside the range go to __dsqrt_rn, as does a
+// failed test.  __dsqrt_rn itself is about twice as many dependent
+// operations, each of which holds a quarter of the FP64 pipe for 64 cycles.
+static __device__ __noinline__ double sqrt_rn_slow(double a) { return __dsqrt_rn(a); }
+__device__ __forceinline__ double sqrt_rn(double a) {
+    const long long ab = dbits(a);
+    const int ea = (int)(ab >> 52) - 1023;  // a > 0
+    if (ea < -500 || ea > 500) return sqrt_rn_slow(a);
+    // f = 2^(ea & 1) 1.m in [1, 4): a = f 4^k
+    const int k = ea >> 1;
+    const float f = __int_as_float(((127 + (ea & 1)) << 23) | (int)((ab >> 29) & 0x7fffff));
+    float r;  // 1 / sqrt(f) in (1/2, 1]
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+    const int rf = __float_as_int(r);
+    const long long yb = ((long long)(((rf >> 23) & 0xff) - 127 - k + 1023) << 52) | ((long long)(rf & 0x7fffff) << 29);
+    const double y = __longlong_as_double(yb);                        // ~ 1 / sqrt(a)
+    const double h = __longlong_as_double(yb - (1LL << 52));          // y / 2
+    const double g = __dmul_rn(a, y);
+    const double c = __fma_rn(-g, h, 0.5);
+    const double g1 = __fma_rn(g, c, g), h1 = __fma_rn(h, c, h);
+    const double s = __fma_rn(__fma_rn(-g1, g1, a), h1, g1);
+    const double e = __fma_rn(-s, s, a);
+    const long long sb = dbits(s);
+    const long long lim = sb + ((long long)((int)(sb >> 52) - 1023 - 52) << 52);  // s ulp(s)
+    if ((sb & 0xfffffffffffffLL) == 0 || (dbits(e) & 0x7fffffffffffffffLL) >= lim) return sqrt_rn_slow(a);
+    return s;
+}
+
+// Right-looking Cholesky D = L L^T in place (lower triangle) on one thread
+// block cluster of C blocks: block b keeps the rows b, b + C, ... in its
+// shared memory (columns 0 .. i of row i are used) and a copy of the whole
+// diagonal.  Column j costs one cluster barrier: one warp of every block takes
+// the pivot's root from its copy of the diagonal, other warps bring the
+// block's own entries of the column up to date, scale them and send them to
+// all blocks; between arriving at the barrier and waiting for it the block
+// finishes the trailing update of column j - 1 (from column j + 1 on).
+//
+// What bounds it.  The trailing updates are n^3 / 3 separately rounded
+// multiply-subtract pairs, 2.7 M FP64 operations for 200 rows, and an SM does
+// two per clock, so one block cannot be fast (1.29 ms for the 2-D p = 3
+// n = 101 hierarchy).  What is left here is the chain of a column: subtract,
+// root, division, exchange.  An FP64 instruction of one warp holds a quarter
+// of the pipe for 64 cycles, so nothing in the chain is computed twice.
+// Measured on that hierarchy: 1.29 -> 0.50 ms; 77 rows 188 -> 155 us.
+// Entries see the same operations in the same order (column after column), so
+// the factor has the same bits.
+constexpr int kCholThreads = 512;
+constexpr int kCholMaxC = 16;
+__global__ void __launch_bounds__(kCholThreads) k_cholesky_cluster(int n, double* D, int* flag) {
+    extern __shared__ double sm[];
+    __shared__ double pivot;
+    uint32_t rank, C;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = kCholThreads >> 5;
+    // [3][n]: columns j - 2, j - 1, j of L (a block ahead writes column j
+    // while one behind still updates with column j - 2)
+    double* lcol = sm;
+    double* diag = sm + 3 * n;  // [n]: the diagonal, up to date past column j - 2
+    double* rows = sm + 4 * n;  // own rows, n entries each, likewise
+    const int own = n > (int)rank ? (n - (int)rank + (int)C - 1) / (int)C : 0;
+    for (int e = tid; e < own * n; e += kCholThreads) {
+        const int u = e / n, k = e - u * n;
+        rows[e] = D[(int64_t)((int)rank + u * (int)C) * n + k];
+    }
+    for (int i = tid; i < n; i += kCholThreads) diag[i] = D[(int64_t)i * n + i];
+    const uint32_t lcol_addr = (uint32_t)__cvta_generic_to_shared(lcol);
+    // every block of the cluster has started before anyone writes its memory
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    __syncthreads();
+    for (int j = 0; j < n; j++) {
+        const double* lp = lcol + ((j + 2) % 3) * n;  // column j - 1
+        const int u0 = j < (int)rank ? 0 : (j - (int)rank) / (int)C + 1;  // first own row > j
+        const int u = u0 + (wid - 1) * 32 + lane;  // this thread's entry of column j (own <= 480 rows: one each)
+        const bool mine = wid > 0 && u < own;
+        const int i = (int)rank + u * (int)C;
+        double v = 0.0;
+        if (wid == 0) {
+            double djj = diag[j];
+            if (j > 0) djj = __dsub_rn(djj, __dmul_rn(lp[j], lp[j]));
+            double piv = 1.0;
+            if (djj > 0.0) piv = sqrt_rn(djj);
+            else if (rank == 0 && lane == 0) atomicOr(flag, 16);
+            if (lane == 0) pivot = piv;
+        } else if (mine) {
+            v = rows[(int64_t)u * n + j];
+            if (j > 0) v = __dsub_rn(v, __dmul_rn(lp[i], lp[j]));
+        }
+        __syncthreads();
+        const double piv = pivot;
+        if (mine) {
+            v = div_rn(v, piv);
+            const uint32_t at = lcol_addr + (uint32_t)((j % 3) * n + i) * 8u;
+            for (uint32_t b = 0; b < C; b++) {
+                uint32_t remote;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(at), "r"(b));
+                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
+            }
+            rows[(int64_t)u * n + j] = v;
+        }
+        if (tid == 0 && j % (int)C == (int)rank) rows[(int64_t)(j / (int)C) * n + j] = piv;
+        // (nothing goes to global memory here: the barrier's release would wait for it)
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        if (j > 0) {  // column j - 1's update from column j + 1 on: a warp per row; the diagonal
+            for (int w = u0 + wid; w < own; w += nw) {
+                const int iw = (int)rank + w * (int)C;
+                double* r = rows + (int64_t)w * n;
+                const double li = lp[iw];
+                for (int k = j + 1 + lane; k < iw; k += 32) r[k] = __dsub_rn(r[k], __dmul_rn(li, lp[k]));
+            }
+            for (int k = j + 1 + tid; k < n; k += kCholThreads) diag[k] = __dsub_rn(diag[k], __dmul_rn(lp[k], lp[k]));
+        }
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        __syncthreads();
+    }
+    for (int e = tid; e < own * n; e += kCholThreads) {
+        const int u = e / n, k = e - u * n, i = (int)rank + u * (int)C;
+        if (k <= i) D[(int64_t)i * n + k] = rows[e];
+    }
+}
+
+// Column c of A^-1 = L^-T L^-1 e_c as below, for factors that fit a block's
+// shared memory (packed lower triangle): a block of four warps per column,
+// its entries in registers (row 128 u + thread), the step's entry passed
+// through shared memory.  An FP64 instruction holds a quarter of the SM's
+// two-lane FP64 pipe for 64 cycles, so a step's updates spread over the four
+// quarters.  Same operations in the same order.  331 -> 155 us on the 2-D
+// p = 3 n = 101 hierarchy.
+constexpr int kInvThreads = 128;
+constexpr int kInvRegs = 2;  // rows per thread: n <= 256, and 8 n + 4 n (n + 1) bytes of shared memory
+__global__ void __launch_bounds__(kInvThreads) k_chol_inverse_smem(int n, const double* __restrict__ L,
+                                                                    double* Ainv) {
+    extern __shared__ double sm[];
+    double* ys = sm;             // [2]: the step's entry, alternating
+    double* rinv = sm + 2;       // [n]
+    double* T = sm + 2 + n;      // row i's columns 0 .. i at i (i + 1) / 2
+    const int tid = threadIdx.x, c = blockIdx.x;
+    for (int i = tid; i < n; i += kInvThreads) rinv[i] = __ddiv_rn(1.0, L[(int64_t)i * n + i]);
+    for (int i = tid >> 5; i < n; i += kInvThreads / 32)
+        for (int k = tid & 31; k <= i; k += 32) T[i * (i + 1) / 2 + k] = L[(int64_t)i * n + k];
+    __syncthreads();
+    double y[kInvRegs];
+#pragma unroll
+    for (int u = 0; u < kInvRegs; u++) y[u] = kInvThreads * u + tid == c ? 1.0 : 0.0;
+    for (int k = c; k < n; k++) {  // forward: L y = e_c
+        if ((k & (kInvThreads - 1)) == tid) {
+            double yk = y[0];
+#pragma unroll
+            for (int u = 1; u < kInvRegs; u++)
+                if (k / kInvThreads == u) yk = y[u];
+            yk = __dmul_rn(yk, rinv[k]);
+            ys[k & 1] = yk;
+#pragma unroll
+            for (int u = 0; u < kInvRegs; u++)
+                if (k / kInvThreads == u) y[u] = yk;
+        }
+        __syncthreads();
+        const double yk = ys[k & 1];
+#pragma unroll
+        for (int u = 0; u < kInvRegs; u++) {
+            const int i = kInvThreads * u + tid;
+            if (i > k && i < n) y[u] = __dsub_rn(y[u], __dmul_rn(T[i * (i + 1) / 2 + k], yk));
+        }
+    }
+    __syncthreads();
+    for (int k = n - 1; k >= 0; k--) {  // backward: L^T x = y
+        if ((k & (kInvThreads - 1)) == tid) {
+            double xk = y[0];
+#pragma unroll
+            for (int u = 1; u < kInvRegs; u++)
+                if (k / kInvThreads == u) xk = y[u];
+            xk = __dmul_rn(xk, rinv[k]);
+            ys[k & 1] = xk;
+#pragma unroll
+            for (int u = 0; u < kInvRegs; u++)
+                if (k / kInvThreads == u) y[u] = xk;
+        }
+        __syncthreads();
+        const double xk = ys[k & 1];
+        const double* row = T + k * (k + 1) / 2;
+#pragma unroll
+        for (int u = 0; u < kInvRegs; u++) {
+            const int i = kInvThreads * u + tid;
+            if (i < k) y[u] = __dsub_rn(y[u], __dmul_rn(row[i], xk));
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kInvRegs; u++)
+        if (kInvThreads * u + tid < n) Ainv[(int64_t)(kInvThreads * u + tid) * n + c] = y[u];
+}
+
+// Right-looking Cholesky D = L L^T in place (lower triangle, one block): the
+// sizes whose rows do not fit a cluster's shared memory.
 __global__ void k_cholesky(int n, double* D, int* flag) {
     __shared__ double piv;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -1819,10 +2021,54 @@ __global__ void k_keep_factor(int n, const double* __restrict__ D, double* L) {
 // in its first n^2 doubles and the factor L (zeros above the diagonal) in
 // the second n^2 (work space of the inverse before).
 cudaError_t launch_dense_spd_inverse(int n, double* D, double* Ainv, int* flag, cudaStream_t s) {
-    k_cholesky<<<AMG_GRID(1), 1024, 0, s>>>(n, D, flag);
-    const size_t sm = sizeof(double) * (size_t)n;  // the diagonal's reciprocals (n <= 4096: 32 KB)
-    if (sm > 48 * 1024) AMG_TRY(cudaFuncSetAttribute(k_chol_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    k_chol_inverse<<<AMG_GRID(blocks_for(n, kWarpsPerBlock, 4096)), kBlock, sm, s>>>(n, D, Ainv, Ainv + (int64_t)n * n);
+    bool done = false;
+    int optin = 0, dev = 0;
+    AMG_TRY(cudaGetDevice(&dev));
+    AMG_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // one cluster where its shared memory holds the rows (16 blocks where the
+    // device schedules such a cluster: n up to about 640; else 8: 450)
+    for (int C = kCholMaxC; C >= 8 && !done; C >>= 1) {
+        const size_t sm = sizeof(double) * (size_t)n * (4 + (n + C - 1) / C);
+        if (sm > (size_t)optin) continue;
+        AMG_TRY(cudaFuncSetAttribute(k_cholesky_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        if (C > 8 && cudaFuncSetAttribute(k_cholesky_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                         cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)C);
+        cfg.blockDim = dim3(kCholThreads);
+        cfg.dynamicSmemBytes = sm;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_cholesky_cluster, &cfg) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();
+            continue;
+        }
+        note_launch();
+        AMG_TRY(cudaLaunchKernelEx(&cfg, k_cholesky_cluster, n, D, flag));
+        done = true;
+    }
+    if (!done) k_cholesky<<<AMG_GRID(1), 1024, 0, s>>>(n, D, flag);
+    const size_t smi = sizeof(double) * (2 + (size_t)n + (size_t)n * (n + 1) / 2);
+    if (n <= kInvThreads * kInvRegs && smi <= (size_t)optin) {
+        AMG_TRY(cudaFuncSetAttribute(k_chol_inverse_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi));
+        k_chol_inverse_smem<<<AMG_GRID(n), kInvThreads, smi, s>>>(n, D, Ainv);
+    } else {
+        const size_t sm = sizeof(double) * (size_t)n;  // the diagonal's reciprocals (n <= 8192: 64 KB)
+        if (sm > 48 * 1024)
+            AMG_TRY(cudaFuncSetAttribute(k_chol_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        k_chol_inverse<<<AMG_GRID(blocks_for(n, kWarpsPerBlock, 4096)), kBlock, sm, s>>>(n, D, Ainv,
+                                                                                        Ainv + (int64_t)n * n);
+    }
     k_keep_factor<<<AMG_GRID(blocks_for((int64_t)n * n, kBlock, 1024)), kBlock, 0, s>>>(n, D, Ainv + (int64_t)n * n);
     return cudaGetLastError();
 }
