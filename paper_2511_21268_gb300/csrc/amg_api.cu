@@ -614,6 +614,7 @@ int build(amg_hierarchy* h, const amg_csr* K) {
         }
         h->nlev = l + 1;
         if (n <= h->o.coarse_max || l + 1 >= h->o.max_levels) break;
+        if (l > 0 && h->o.mpnn_weights) RC(mpnn_setup_level(h, l));
         if (l == 0) {
             RC(dalloc(h, &F.w, n));
             double* wt;

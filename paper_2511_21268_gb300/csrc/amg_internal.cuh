@@ -323,6 +323,7 @@ int multi_part_slots();
 // mpnn.cu
 void mpnn_free(amg_hierarchy* h);
 int mpnn_setup_fork(amg_hierarchy* h);
+int mpnn_setup_level(amg_hierarchy* h, int l);
 int mpnn_setup_join(amg_hierarchy* h);
 int mpnn_setup_theta(amg_hierarchy* h);
 // stream_kernels.cu
