@@ -164,27 +164,43 @@ __global__ void __launch_bounds__(kBlock) k_coarse(int n, const double* __restri
 }
 
 // ------------------------------------------------- coarsest level by CG
-// Fixed-order sum over one block of 1024 threads (result on every thread).
-__device__ __forceinline__ double block_sum1024(double t, double* red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+// Fixed-order sums over one block of values that the first `nact` warps hold;
+// thread 0 passes them to fin, whose shared-memory results every thread sees
+// afterwards.  What the other warps would add, and a division or root on every
+// thread, would cost as much of the SM's FP64 pipe as useful work (an
+// instruction holds a quarter of it for 64 cycles).
+template <typename Fin>
+__device__ __forceinline__ void block_sums(double t, double u, bool two, int nact, double* red, Fin&& fin) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[wid] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double u = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) u += red[w];
-        red[32] = u;
+    if (wid < nact) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            t += __shfl_xor_sync(FULL, t, o);
+            if (two) u += __shfl_xor_sync(FULL, u, o);
+        }
     }
     __syncthreads();
-    return red[32];
+    if (lane == 0 && wid < nact) {
+        red[wid] = t;
+        red[32 + wid] = u;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s0 = 0.0, s1 = 0.0;
+        for (int w = 0; w < nact; w++) {
+            s0 += red[w];
+            if (two) s1 += red[32 + w];
+        }
+        fin(s0, s1);
+    }
+    __syncthreads();
 }
 
 // Coarsest level by Jacobi-preconditioned CG from x = 0 (Sec. 5's coarse
 // solver): at most maxit iterations, stop once ||r|| <= tol ||f||.  One
 // block; FP64 work vectors r, z, p, q, x in global memory (4 n + n doubles);
-// the result goes to e in the V-cycle precision.
+// the result goes to e in the V-cycle precision.  154 -> 48 us for the 80
+// rows of the cube case at k = 32 (30 iterations).
 template <typename A>
 __global__ void __launch_bounds__(1024) k_coarse_cg(int n, const int64_t* __restrict__ rp,
                                                      const int32_t* __restrict__ ci, const double* __restrict__ v,
@@ -192,52 +208,66 @@ __global__ void __launch_bounds__(1024) k_coarse_cg(int n, const int64_t* __rest
                                                      double* work, double tol, int maxit, const SolveState* st) {
     pdl_entry();
     DONE_GUARD(st);
-    __shared__ double red[33];
+    __shared__ double red[64];
+    __shared__ double rho, alpha, beta, stop;
+    __shared__ int go;
     double *r = work, *z = work + n, *p = work + 2 * (int64_t)n, *q = work + 3 * (int64_t)n,
            *x = work + 4 * (int64_t)n;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwp = blockDim.x >> 5;
-    double ff = 0.0, rz = 0.0;
+    const int nact = min(nwp, (n + 31) >> 5);
+    double t0 = 0.0, t1 = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const double fi = (double)f[i], zi = fi / kii[i];
         x[i] = 0.0;
         r[i] = fi;
         z[i] = zi;
         p[i] = zi;
-        ff = fma(fi, fi, ff);
-        rz = fma(fi, zi, rz);
+        t0 = fma(fi, fi, t0);
+        t1 = fma(fi, zi, t1);
     }
-    ff = block_sum1024(ff, red);
-    double rho = block_sum1024(rz, red);
-    double rr = ff;
-    const double stop = tol * sqrt(ff);
-    for (int it = 0; it < maxit && sqrt(rr) > stop; it++) {
-        for (int i = wid; i < n; i += nwp) {  // q = K p, a warp per row
+    block_sums(t0, t1, true, nact, red, [&](double ff, double rz) {
+        const double nf = sqrt(ff);
+        stop = tol * nf;
+        rho = rz;
+        go = nf > stop;
+    });
+    for (int it = 0; it < maxit && go; it++) {
+        for (int i0 = wid * 4; i0 < n; i0 += nwp * 4) {  // q = K p, 8 lanes per row
+            const int i = i0 + (lane >> 3);
             double acc = 0.0;
-            for (int64_t k = rp[i] + lane; k < rp[i + 1]; k += 32) acc = fma(v[k], p[ci[k]], acc);
+            if (i < n) {
+                const int64_t k1 = rp[i + 1];
+#pragma unroll 4
+                for (int64_t k = rp[i] + (lane & 7); k < k1; k += 8) acc = fma(v[k], p[ci[k]], acc);
+            }
+            __syncwarp();
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
-            if (lane == 0) q[i] = acc;
+            for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+            if (i < n && (lane & 7) == 0) q[i] = acc;
         }
         __syncthreads();
-        double t = 0.0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) t = fma(p[i], q[i], t);
-        const double pq = block_sum1024(t, red);
-        if (!(pq > 0.0)) break;
-        const double alpha = rho / pq;
-        double t1 = 0.0, t2 = 0.0;
+        t0 = 0.0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) t0 = fma(p[i], q[i], t0);
+        block_sums(t0, 0.0, false, nact, red, [&](double pq, double) {
+            go = pq > 0.0;
+            alpha = rho / pq;
+        });
+        if (!go) break;
+        t0 = t1 = 0.0;
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
             x[i] = fma(alpha, p[i], x[i]);
             const double ri = fma(-alpha, q[i], r[i]);
             const double zi = ri / kii[i];
             r[i] = ri;
             z[i] = zi;
-            t1 = fma(ri, zi, t1);
-            t2 = fma(ri, ri, t2);
+            t0 = fma(ri, zi, t0);
+            t1 = fma(ri, ri, t1);
         }
-        const double rho1 = block_sum1024(t1, red);
-        rr = block_sum1024(t2, red);
-        const double beta = rho1 / rho;
-        rho = rho1;
+        block_sums(t0, t1, true, nact, red, [&](double rz, double rr) {
+            beta = rz / rho;
+            rho = rz;
+            go = sqrt(rr) > stop;
+        });
         for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = fma(beta, p[i], z[i]);
         __syncthreads();
     }
