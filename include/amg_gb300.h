@@ -524,10 +524,13 @@ int amg_iga_size(const amg_iga_patch* P, int64_t* n, int64_t* nnz);
  * amg_iga_size gives, owned by the caller -- on cuda_stream (NULL = legacy
  * default stream) of the current device; returns after the work finished.
  * Device workspace is taken from the library's stream-ordered pool and
- * released before the return: at its peak 8 (4 R Q^2 + 4 R^2 Q) bytes with
- * Q = n nq and R = (2p+1) m (2.7 GB for n = 64, p = 3; 8.9 GB for n = 96),
- * plus 8 Q^2 (2M rounded up to 16) for kappa.  *flops (may be NULL) receives the
- * floating-point operations of the quadrature sums (2 per multiply-add).
+ * released before the return: at its peak 8 (4 S Q^2 + 4 S R Q) bytes with
+ * Q = n nq, R = (2p+1) m and S = (p+1) m (1.5 GB for n = 64, p = 3; 5.1 GB
+ * for n = 96), and before that 40 Q^3 bytes of coefficients with, for kappa,
+ * about 100 MB (at least 1024 bytes per feature column, 2M rounded up to 32) and 16 Q
+ * bytes per feature column.  *flops (may be NULL) receives the floating-point
+ * operations of the quadrature sums of all stored entries (2 per
+ * multiply-add; K's symmetry halves what runs).
  * Returns AMG_OK, AMG_ERR_ARG, AMG_ERR_NOMEM or AMG_ERR_CUDA. */
 int amg_iga_assemble(const amg_iga_patch* P, int64_t* rowptr, int32_t* col, double* val, double* F,
                      void* cuda_stream, double* flops);

@@ -1,7 +1,7 @@
 """The coefficient's fixed-point product at the edges of its tiles: numbers of
 features around multiples of 16 (columns padded to 32), Gauss points that are
-no multiple of 64, more features than one piece of the plane holds; and
-values that are not finite.  Entries within 1e-12 of the oracle's element loop
+no multiple of 64, more features than one piece of the plane holds; K's
+exact symmetry; and values that are not finite.  Entries within 1e-12 of the oracle's element loop
 (relative to the largest), as in test_gpu_assembly.py."""
 import math
 
@@ -37,6 +37,7 @@ def test_values_match_the_element_loop(n, p, nq, M):
     for i in range(g["n"]):
         D[i, ci[rp[i]:rp[i + 1]]] = v[rp[i]:rp[i + 1]]
     assert np.abs(D - K).max() <= 1e-12 * np.abs(K).max()
+    assert np.array_equal(D, D.T)  # each pair of entries is computed once
     assert np.abs(g["F"].cpu().numpy() - F).max() <= 1e-12 * np.abs(F).max()
 
 
