@@ -395,14 +395,28 @@ __global__ void __launch_bounds__(kBlock) k_nn_in_bwd(int n, const float* __rest
     for (int f = 0; f < 5; f++) block_lane_sum(red, g[f], out + f * H);
 }
 
-// gacc[dst[t]] += sum over blocks (in block order, FP64) of slot t
-__global__ void k_nn_grad_sum(int nblocks, const float* __restrict__ part, int count, const int* __restrict__ dst,
-                              double* __restrict__ gacc) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count) return;
+// gacc[dst[t]] += sum over blocks (FP64, fixed order) of slot t.  A block per
+// 32 slots, a warp per eighth of the block partials: the conversions and adds
+// run on 65 SMs' FP64 pipes with 32 in a chain, instead of on 9 with 256
+// (20 -> 6 us for a dense layer).
+constexpr int kSumWarps = 8;
+__global__ void __launch_bounds__(32 * kSumWarps) k_nn_grad_sum(int nblocks, const float* __restrict__ part,
+                                                                 int count, const int* __restrict__ dst,
+                                                                 double* __restrict__ gacc) {
+    __shared__ double sh[kSumWarps][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = blockIdx.x * 32 + lane;
+    const int b0 = wid * nblocks / kSumWarps, b1 = (wid + 1) * nblocks / kSumWarps;
     double s = 0.0;
-    for (int b = 0; b < nblocks; b++) s += (double)part[(int64_t)b * kGradSlots + t];
-    gacc[dst[t]] += s;
+    if (t < count) {
+#pragma unroll 8
+        for (int b = b0; b < b1; b++) s += (double)part[(int64_t)b * kGradSlots + t];
+    }
+    sh[wid][lane] = s;
+    __syncthreads();
+    if (wid == 0 && t < count) {
+        for (int w = 1; w < kSumWarps; w++) s += sh[w][lane];
+        gacc[dst[t]] += s;
+    }
 }
 
 // ------------------------------------------------ damped V-cycle (FP64)
@@ -1047,22 +1061,22 @@ cudaError_t net_backward(amg_hierarchy* h, const float* wd, int l, const double*
     float *u0 = m.t[0], *h0 = m.t[1], *m1 = m.t[2], *u1 = m.t[3], *h1 = m.t[4], *m2 = m.t[5], *u2 = m.t[6],
           *h2 = m.t[7];
     float *b0 = w.bw[0], *b1 = w.bw[1], *b2 = w.bw[2];
-    const int gs = eblk(kGradSlots);
+    const int gs = (kGradSlots + 31) / 32;
     k_nn_out_bwd<<<AMG_GRID(gg), kBlock, 0, s>>>(n, wd, m.domega, m.sg, h2, u2, b0, w.part, m.cap, dtheta, m.sgt);
-    k_nn_grad_sum<<<AMG_GRID(gs), kBlock, 0, s>>>(gg, w.part, 2 * H + 2, w.dst, w.gacc);
+    k_nn_grad_sum<<<AMG_GRID(gs), 32 * kSumWarps, 0, s>>>(gg, w.part, 2 * H + 2, w.dst, w.gacc);
     // layer 2: du2 (b0) -> dm2 (b1), V2^T du2 (b2); dh1 = A' dm2 + V2^T du2 (b0)
     k_nn_dense_bwd<<<AMG_GRID(gg), kBlock, 0, s>>>(n, wd, 2, b0, m2, h1, b1, b2, w.part);
-    k_nn_grad_sum<<<AMG_GRID(gs), kBlock, 0, s>>>(gg, w.part, 2 * H * H + H, w.dst + kGradSlots, w.gacc);
+    k_nn_grad_sum<<<AMG_GRID(gs), 32 * kSumWarps, 0, s>>>(gg, w.part, 2 * H * H + H, w.dst + kGradSlots, w.gacc);
     k_nn_spmm<<<AMG_GRID(g), kBlock, 0, s>>>(n, L.A.rowptr, L.A.col, m.ap, b1, b2, b0);
     k_nn_relu_mask<<<AMG_GRID(eblk(cnt)), kBlock, 0, s>>>(cnt, u1, b0);
     // layer 1
     k_nn_dense_bwd<<<AMG_GRID(gg), kBlock, 0, s>>>(n, wd, 1, b0, m1, h0, b1, b2, w.part);
-    k_nn_grad_sum<<<AMG_GRID(gs), kBlock, 0, s>>>(gg, w.part, 2 * H * H + H, w.dst + 2 * kGradSlots, w.gacc);
+    k_nn_grad_sum<<<AMG_GRID(gs), 32 * kSumWarps, 0, s>>>(gg, w.part, 2 * H * H + H, w.dst + 2 * kGradSlots, w.gacc);
     k_nn_spmm<<<AMG_GRID(g), kBlock, 0, s>>>(n, L.A.rowptr, L.A.col, m.ap, b1, b2, b0);
     k_nn_relu_mask<<<AMG_GRID(eblk(cnt)), kBlock, 0, s>>>(cnt, u0, b0);
     // input layer
     k_nn_in_bwd<<<AMG_GRID(gg), kBlock, 0, s>>>(n, b0, m.x, w.part);
-    k_nn_grad_sum<<<AMG_GRID(gs), kBlock, 0, s>>>(gg, w.part, 5 * H, w.dst + 3 * kGradSlots, w.gacc);
+    k_nn_grad_sum<<<AMG_GRID(gs), 32 * kSumWarps, 0, s>>>(gg, w.part, 5 * H, w.dst + 3 * kGradSlots, w.gacc);
     return cudaGetLastError();
 }
 
@@ -1476,21 +1490,32 @@ int amg_mpnn_train(amg_hierarchy* const* hs, int32_t count, float* w, int32_t st
     MP_RC(sync_status(h0));
     for (int t = 0; t < steps; t++) {
         double lsum = 0.0;
-        // every hierarchy's loss and gradient with the same weights (its own
-        // stream, waited for on the host before the weights change)
-        for (int k = 0; k < count; k++) {
-            if (twogrid_theta(hs[k]))
-                MP_RC(theta_loss_grad_enqueue(hs[k], w, nprobe, seed + (uint64_t)t));
-            else
-                MP_RC(loss_grad_enqueue(hs[k], w, nprobe, seed + (uint64_t)t));
-            int bad = 0;
+        // every hierarchy's loss and gradient with the same weights: enqueued
+        // on all their streams first, which then run side by side, and waited
+        // for on the host before the weights change (also before an error
+        // returns)
+        int queued = 0, rc = AMG_OK;
+        for (; queued < count && rc == AMG_OK; queued++)
+            rc = twogrid_theta(hs[queued]) ? theta_loss_grad_enqueue(hs[queued], w, nprobe, seed + (uint64_t)t)
+                                           : loss_grad_enqueue(hs[queued], w, nprobe, seed + (uint64_t)t);
+        const int good = rc == AMG_OK ? queued : queued - 1;
+        int first = AMG_OK;  // the first hierarchy's error
+        for (int k = 0; k < queued; k++) {
+            int bad = 0, r = AMG_OK;
             double lk = 0.0;
-            MP_RC(read_host(hs[k], hs[k]->mp->bad, &bad));
-            if (bad) return AMG_ERR_BREAKDOWN;
-            MP_RC(read_host(hs[k], hs[k]->mp->loss, &lk));
-            if (!isfinite(lk)) return AMG_ERR_NAN;
+            if (k < good) {
+                r = read_host(hs[k], hs[k]->mp->bad, &bad);
+                if (r == AMG_OK && bad) r = AMG_ERR_BREAKDOWN;
+                if (r == AMG_OK) r = read_host(hs[k], hs[k]->mp->loss, &lk);
+                if (r == AMG_OK && !isfinite(lk)) r = AMG_ERR_NAN;
+            } else {
+                sync_status(hs[k]);
+                r = rc;
+            }
+            if (first == AMG_OK) first = r;
             lsum += lk;
         }
+        if (first != AMG_OK) return first;
         // mean gradient (fixed hierarchy order), then one Adam step
         for (int k = 0; k < count; k++)
             k_scale_add<<<AMG_GRID(eblk(AMG_MPNN_NPARAM)), kBlock, 0, h0->s>>>(
