@@ -9,8 +9,9 @@
 // Coarsening stops at coarse_max rows, on stagnation or at max_levels; the
 // coarsest matrix is inverted densely.
 //
-// Solve: the CG start phase is launched directly, the iterations run as a
-// captured CUDA graph of kGraphIters iterations whose kernels turn into
+// Solve: small FP64 systems run as one kernel on one cluster
+// (cluster_solve.cu); else the CG start phase is launched directly, the
+// iterations run as a captured CUDA graph of kGraphIters iterations whose kernels turn into
 // no-ops once the device-side state says "done"; the host reads the state
 // once per graph launch.
 #include <cuda_runtime.h>
@@ -1141,9 +1142,20 @@ int amg_setup_batch(int32_t count, const amg_csr* Ks, const amg_opts* opts, void
 static int run_solve(amg_hierarchy* h, int32_t* iters) {
     cudaStream_t s = h->s;
     CK(cudaEventRecord(h->ev0, s));
-    CK(enqueue_pcg_start(h, s));
     h->info.graph_build_ms = 0.0;
-    if (!h->graph) {
+    // small systems: one kernel on one cluster
+    bool cluster = cluster_solve_blocks(h) > 0;
+    if (cluster) {
+        CK(launch_cluster_pcg(h, 1));
+        CK(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (h->st_host->status == kClusterUnfit) {
+            h->cluster_blocks = 0;
+            cluster = false;
+        }
+    }
+    if (!cluster) CK(enqueue_pcg_start(h, s));
+    if (!cluster && !h->graph) {
         const auto tb0 = std::chrono::steady_clock::now();
         cudaGraph_t g;
         const long long before = amg::g_launches.load();
@@ -1169,11 +1181,13 @@ static int run_solve(amg_hierarchy* h, int32_t* iters) {
         h->info.graph_build_ms =
             std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tb0).count();
     }
-    const int max_launches = h->itmax / kGraphIters + 2;
+    const int max_launches = h->itmax / (cluster ? cluster_solve_iters() : kGraphIters) + 2;
     int it_before = 0;
     for (int k = 0; k <= max_launches + 1; k++) {
-        CK(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
+        if (!cluster || k > 0) {
+            CK(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+        }
         if (h->prof && k > 0) {  // accumulate the kernels of the launch that just finished
             const int ndone = h->st_host->iters - it_before;
             for (int j = 0; j < kGraphIters; j++)
@@ -1189,6 +1203,10 @@ static int run_solve(amg_hierarchy* h, int32_t* iters) {
         }
         it_before = h->st_host->iters;
         if (h->st_host->done || k > max_launches) break;
+        if (cluster) {
+            CK(launch_cluster_pcg(h, 0));
+            continue;
+        }
         CK(cudaGraphLaunch(h->graph, s));
         amg::g_launches += h->graph_kernels;
     }

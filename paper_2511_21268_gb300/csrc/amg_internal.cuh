@@ -230,6 +230,8 @@ struct amg_hierarchy {
     double tune_ms = 0.0;  // host time of the setup's autotuning (0 when skipped or cached)
     int galerkin_spgemm_passes = 0;  // pass Galerkin products done by the SpGEMM path (too-wide rows)
     int sell64_warps = 0;  // warps per block of those passes
+    int cluster_blocks = -1;  // blocks of the one-cluster solve (0: none, -1: not asked yet)
+    int cluster_smem = 0;     // and their dynamic shared memory
     // multi-system solves
     amg::MultiWork* mw = nullptr;
     // learned smoother damping: network buffers, and whether the smoother
@@ -314,6 +316,11 @@ cudaError_t enqueue_pcg_iteration(amg_hierarchy* h, cudaStream_t s);
 cudaError_t launch_final_residual(amg_hierarchy* h, cudaStream_t s);
 cudaError_t launch_rowgroup_pq(amg_hierarchy* h, cudaStream_t s, bool batch = false);
 double* final_residual_slot(amg_hierarchy* h);
+// cluster_solve.cu: CG of a small system as one kernel on one cluster
+constexpr int kClusterUnfit = 1;             // SolveState::status: its rows do not fit the blocks
+int cluster_solve_blocks(amg_hierarchy* h);  // 0: does not apply
+int cluster_solve_iters();                   // iterations of one launch
+cudaError_t launch_cluster_pcg(amg_hierarchy* h, int start);
 // multi_solve.cu
 cudaError_t enqueue_multi_start(amg_hierarchy* h, cudaStream_t s);
 cudaError_t enqueue_multi_iteration(amg_hierarchy* h, cudaStream_t s);
