@@ -715,6 +715,8 @@ static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s, bool rows_only 
         Level& C = h->lev[l + 1];
         const int n = F.A.n;
         const int rpw = level_rows(h, F, rows_only), nb = row_blocks(n, rpw);
+        const bool coarsest = (l + 1 == L - 1);
+        bool restricted = false;
         Vw::vals(F, l, rpw, [&](auto mat) {
             using M = decltype(mat);
             auto sweep_and_resid = [&](auto fp) {
@@ -751,14 +753,26 @@ static cudaError_t vcycle_impl(amg_hierarchy* h, cudaStream_t s, bool rows_only 
                     }
                 }
                 with_rpw<M>(rpw, [&](auto R) {
-                    launch_pdl(k_resid<decltype(R)::value, A, M, FT, A>, nb, kBlock, 0, s, n, mat, fp, xc, rb, st);
+                    constexpr int RPW = decltype(R)::value;
+                    if constexpr (RPW == 1 || RPW == 4) {
+                        if (!F.smoothed) {
+                            // coarse rows of a block: its warps' share of members
+                            const int rows = std::max(1, RPW * kWarpsPerBlock >> F.npass);
+                            launch_pdl(k_resid_restrict<RPW, A, M, FT>, (C.A.n + rows - 1) / rows, kBlock, 0, s,
+                                       C.A.n, rows, mat, fp, xc, Vw::invd(C), F.mem_ptr, F.mem_idx, F.pval, Vw::f(C),
+                                       coarsest ? nullptr : xcur[l + 1], st);
+                            restricted = true;
+                            return;
+                        }
+                    }
+                    launch_pdl(k_resid<RPW, A, M, FT, A>, nb, kBlock, 0, s, n, mat, fp, xc, rb, st);
                 });
                 if (l == 0) prof_mark(h, 1, 1, s);
             };
             if (l == 0) sweep_and_resid(static_cast<const double*>(h->r));
             else sweep_and_resid(static_cast<const A*>(Vw::f(F)));
         });
-        const bool coarsest = (l + 1 == L - 1);
+        if (restricted) continue;
         if (F.smoothed)  // f_c = P_bar^T r
             sp_restrict<A>(F, C, xalt[l], Vw::f(C), coarsest ? nullptr : xcur[l + 1], Vw::invd(C), st, s);
         else
