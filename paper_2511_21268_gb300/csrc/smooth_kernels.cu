@@ -134,6 +134,17 @@ __device__ __forceinline__ int64_t chunk_item(int f, int64_t q0, int len, int in
     return qs + (f - (is - ls));
 }
 
+// Marks column J.  Most items of a row meet a column that is marked already
+// (some 300 B rows of 100 to 150 entries share 1,000 columns or so), and the
+// lanes of a warp that meet one word would take turns at its atomic: a read
+// spares it.  A read of an old word costs one atomic more.  The counting passes
+// of the paper's cube, p = 3, k = 32: 8.8 -> 4.7 ms, its last product (which
+// marks its rows in the numeric pass too) 6.7 -> 6.1 ms.
+__device__ __forceinline__ void set_bit(uint32_t* bits, int J) {
+    const uint32_t m = 1u << (J & 31);
+    if (!(*(volatile uint32_t*)&bits[J >> 5] & m)) atomicOr(&bits[J >> 5], m);
+}
+
 // Marks the output columns of row i (A's row [a0, a1)) in bits (span from lo).
 __device__ __forceinline__ void mark_row(const int32_t* __restrict__ aci, const int64_t* __restrict__ brp,
                                          const int32_t* __restrict__ bci, int64_t a0, int64_t a1, int lo, int lane,
@@ -154,7 +165,7 @@ __device__ __forceinline__ void mark_row(const int32_t* __restrict__ aci, const 
             }
 #pragma unroll
             for (int u = 0; u < kSpBatch; u++)
-                if (J[u] >= 0) atomicOr(&bits[J[u] >> 5], 1u << (J[u] & 31));
+                if (J[u] >= 0) set_bit(bits, J[u]);
         }
     }
 }
@@ -368,7 +379,7 @@ __global__ void __launch_bounds__(BT) k_sp_row_blk(int n, const int64_t* __restr
                     }
 #pragma unroll
                     for (int u = 0; u < kSpUnroll; u++)
-                        if (J[u] >= 0) atomicOr(&bits[J[u] >> 5], 1u << (J[u] & 31));
+                        if (J[u] >= 0) set_bit(bits, J[u]);
                 }
             }
         }
