@@ -1319,7 +1319,8 @@ static int ensure_multi(amg_hierarchy* h, int R, int S, const int32_t* seg) {
     RC(walloc(h, *w, &w->st, (size_t)S));
     RC(walloc(h, *w, &w->active, 1));
     RC(walloc(h, *w, &w->params, 2));
-    RC(walloc(h, *w, &w->due, 1));
+    RC(walloc(h, *w, &w->due, 2));
+    CK(cudaMemsetAsync(w->due, 0, 2 * sizeof(unsigned), h->s));
     w->R = R;  // complete: a failed attempt is built again
     return AMG_OK;
 }

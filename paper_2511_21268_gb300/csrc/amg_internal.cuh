@@ -66,7 +66,8 @@ struct MultiWork {
     MultiState* st = nullptr;
     int* active = nullptr;    // systems still iterating
     int* params = nullptr;    // itmax, replacement period
-    unsigned* due = nullptr;  // right-hand sides (batch: any) whose residual replacement is due
+    unsigned* due = nullptr;  // [0]: right-hand sides (batch: any) whose residual replacement is due; [1]: blocks done with
+                              // the scalars (0 between kernels)
     void* lf[AMG_MAX_LEVELS] = {};
     void* lx[AMG_MAX_LEVELS] = {};
     void* lt[AMG_MAX_LEVELS] = {};

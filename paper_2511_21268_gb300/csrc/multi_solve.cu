@@ -738,77 +738,69 @@ struct Parts {
     const int* tile0;
 };
 
-// tot[s] = sum of system s's partials, in a fixed order, for s < S (shared
-// memory; one block).  Right-hand sides: the block's threads split the block
-// partials of each column; batch: a warp per system.
-__device__ void sum_systems(const Parts& P, int S, const double* __restrict__ part, double* tot, double* sh) {
-    if (!P.tile0) {
-        const int per = blockDim.x / P.Rs, c = threadIdx.x % P.Rs, j = threadIdx.x / P.Rs;
-        double s = 0.0;
-        if (j < per) {
+// Scalar kernels: a warp per system, kScalSys systems per block.  An FP64
+// instruction of a warp holds a quarter of an SM's pipe for 64 cycles: 304
+// partials of 16 columns in one block are 2.4 us of adds, on four SMs a quarter.
+// Measured, 16 right-hand sides: alpha 11.1 -> 8.1 us, beta 11.3 -> 8.4, the
+// convergence test 7.6 -> 6.9; a batch of 16: 6.6 -> 4.6, 7.1 -> 5.0, 5.5 -> 4.5.
+constexpr int kScalSys = 4;
+
+// Sum of system s's partials on every lane of the warp, in a fixed order.
+__device__ __forceinline__ double sum_system(const Parts& P, int s, const double* __restrict__ part, int lane) {
+    const int k0 = P.tile0 ? P.tile0[s] : 0, k1 = P.tile0 ? P.tile0[s + 1] : P.nb;
+    const int64_t step = P.tile0 ? 1 : P.Rs;
+    const double* __restrict__ p = P.tile0 ? part : part + s;
+    double t = 0.0;
 #pragma unroll 8
-            for (int b = j; b < P.nb; b += per) s += part[(int64_t)b * P.Rs + c];
-        }
-        __syncthreads();
-        sh[threadIdx.x] = s;
-        // column c's `per` values, folded in half until one is left
-        for (int w = per; w > 1;) {
-            const int half = (w + 1) >> 1;
-            __syncthreads();
-            if (j + half < w) sh[threadIdx.x] += sh[threadIdx.x + half * P.Rs];
-            w = half;
-        }
-        __syncthreads();
-        if ((int)threadIdx.x < S) tot[threadIdx.x] = sh[threadIdx.x];
-    } else {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        __syncthreads();
-        for (int s = wid; s < S; s += nw) {
-            double t = 0.0;
-            for (int k = P.tile0[s] + lane; k < P.tile0[s + 1]; k += 32) t += part[k];
+    for (int k = k0 + lane; k < k1; k += 32) t += p[k * step];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-            if (lane == 0) tot[s] = t;
-        }
-    }
-    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+    return t;
 }
 
-constexpr int kScalThreads = 1024;
-#define SCAL_SHARED                      \
-    __shared__ double sh[kScalThreads]; \
-    __shared__ double t0[kScalThreads];
+#define SCAL_SYSTEM                    \
+    const int lane = threadIdx.x & 31; \
+    const int s = blockIdx.x * kScalSys + ((int)threadIdx.x >> 5);
 
-// *active = number of systems not done (0 as well once the single-system
-// state, which the batch's V-cycle kernels read, says stop).
-__device__ void count_active(int S, const MultiState* st, int* active, SolveState* single) {
+// In the block that gets here last: *active = number of systems not done (0 as
+// well once the single-system state, which the batch's V-cycle kernels read,
+// says stop).  `ticket` is zero again afterwards.
+__device__ void count_active(int S, const MultiState* st, int* active, unsigned* ticket, SolveState* single,
+                             unsigned* clear = nullptr) {
     __shared__ int cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) cnt = 0;
-    __syncthreads();
-    for (int s = threadIdx.x; s < S; s += blockDim.x)
-        if (!st[s].done) atomicAdd(&cnt, 1);
+    __shared__ bool last;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const int a = single->done ? 0 : cnt;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last) *ticket = 0;
+        __threadfence();
+        cnt = 0;
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int k = threadIdx.x; k < S; k += blockDim.x)
+        if (!__ldcg(&st[k].done)) atomicAdd(&cnt, 1);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const int a = __ldcg(&single->done) ? 0 : cnt;
         *active = a;
         if (a == 0) single->done = 1;
+        if (clear) *clear = 0;
     }
 }
 
 // all systems' squared norms of the start residual and of F
-__global__ void __launch_bounds__(kScalThreads) k_m_scal_init(Parts P, int S, const double* part_rr,
+__global__ void __launch_bounds__(kScalSys * 32) k_m_scal_init(Parts P, int S, const double* part_rr,
                                                                const double* part_ff, double rtol, int itmax,
                                                                int repl, MultiState* st, int* active, int* itmax_out,
                                                                unsigned* due, SolveState* single) {
     pdl_entry();
-    SCAL_SHARED
-    __shared__ double t1[kScalThreads];
-    sum_systems(P, S, part_rr, t0, sh);
-    sum_systems(P, S, part_ff, t1, sh);
-    for (int s = threadIdx.x; s < S; s += blockDim.x) {
+    SCAL_SYSTEM
+    const double rr = s < S ? sum_system(P, s, part_rr, lane) : 0.0, ff = s < S ? sum_system(P, s, part_ff, lane) : 0.0;
+    if (s < S && lane == 0) {
         MultiState& m = st[s];
-        const double nF = sqrt(t1[s]), nr = sqrt(t0[s]);
+        const double nF = sqrt(ff), nr = sqrt(rr);
         m.nF = nF;
         m.tol = rtol * nF;
         m.nr = nr;
@@ -826,142 +818,135 @@ __global__ void __launch_bounds__(kScalThreads) k_m_scal_init(Parts P, int S, co
             m.done = 1;
         }
     }
-    if (threadIdx.x == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         itmax_out[0] = itmax;
         itmax_out[1] = repl;
-        *due = 0;
+        due[0] = 0;
         single->done = 0;
         single->status = AMG_OK;
     }
-    count_active(S, st, active, single);
+    count_active(S, st, active, due + 1, single);
 }
 
-__global__ void __launch_bounds__(kScalThreads) k_m_scal_alpha(Parts P, int S, const double* part_pq,
+__global__ void __launch_bounds__(kScalSys * 32) k_m_scal_alpha(Parts P, int S, const double* part_pq,
                                                                 const double* part_pr, int flexible, MultiState* st,
-                                                                int* active, SolveState* single) {
+                                                                int* active, unsigned* due, SolveState* single) {
     pdl_entry();
     if (*active == 0) return;
-    SCAL_SHARED
-    __shared__ double t1[kScalThreads];
-    sum_systems(P, S, part_pq, t0, sh);
-    if (flexible) sum_systems(P, S, part_pr, t1, sh);
-    for (int s = threadIdx.x; s < S; s += blockDim.x) {
-        MultiState& m = st[s];
-        if (m.done) continue;
-        const double pq = t0[s];
-        const double num = flexible ? t1[s] : m.rho;
-        m.pq = pq;
-        if (!(pq > 0.0)) {
-            m.status = (isnan(pq) || isnan(num)) ? AMG_ERR_NAN : AMG_ERR_BREAKDOWN;
-            m.done = 1;
-        } else {
-            m.alpha = num / pq;
+    SCAL_SYSTEM
+    if (s < S && !st[s].done) {
+        const double pq = sum_system(P, s, part_pq, lane);
+        const double num = flexible ? sum_system(P, s, part_pr, lane) : st[s].rho;
+        if (lane == 0) {
+            MultiState& m = st[s];
+            m.pq = pq;
+            if (!(pq > 0.0)) {
+                m.status = (isnan(pq) || isnan(num)) ? AMG_ERR_NAN : AMG_ERR_BREAKDOWN;
+                m.done = 1;
+            } else {
+                m.alpha = num / pq;
+            }
         }
     }
-    count_active(S, st, active, single);
+    count_active(S, st, active, due + 1, single);
 }
 
 // *due: the right-hand sides (bit s) whose FP64 residual replacement is due;
-// nonzero for a batch when any system's is.
-__global__ void __launch_bounds__(kScalThreads) k_m_scal_conv(Parts P, int S, const double* part_rr, int mixed,
+// nonzero for a batch when any system's is (zero before).
+__global__ void __launch_bounds__(kScalSys * 32) k_m_scal_conv(Parts P, int S, const double* part_rr, int mixed,
                                                                const int* params, MultiState* st, int* active,
                                                                unsigned* due, SolveState* single) {
     pdl_entry();
     if (*active == 0) return;
-    SCAL_SHARED
-    __shared__ unsigned mask;
-    if (threadIdx.x == 0) mask = 0;
-    sum_systems(P, S, part_rr, t0, sh);
-    const int itmax = params[0], repl = params[1];
-    for (int s = threadIdx.x; s < S; s += blockDim.x) {
-        MultiState& m = st[s];
-        if (m.done) continue;
-        const double nr = sqrt(t0[s]);
-        const int it = m.iters + 1;
-        m.iters = it;
-        m.nr = nr;
-        if (isnan(nr) || isinf(nr)) {
-            m.status = AMG_ERR_NAN;
-            m.done = 1;
-        } else if (mixed && (nr <= m.tol || it >= itmax || (repl > 0 && it % repl == 0))) {
-            m.replace_now = 1;
-            atomicOr(&mask, 1u << (s & 31));
-        } else if (nr <= m.tol) {
-            m.done = 1;
-        } else if (it >= itmax) {
-            m.status = AMG_ERR_NOT_CONVERGED;
-            m.done = 1;
+    SCAL_SYSTEM
+    if (s < S && !st[s].done) {
+        const double rr = sum_system(P, s, part_rr, lane);
+        if (lane == 0) {
+            MultiState& m = st[s];
+            const int itmax = params[0], repl = params[1];
+            const double nr = sqrt(rr);
+            const int it = m.iters + 1;
+            m.iters = it;
+            m.nr = nr;
+            if (isnan(nr) || isinf(nr)) {
+                m.status = AMG_ERR_NAN;
+                m.done = 1;
+            } else if (mixed && (nr <= m.tol || it >= itmax || (repl > 0 && it % repl == 0))) {
+                m.replace_now = 1;
+                atomicOr(due, 1u << (s & 31));
+            } else if (nr <= m.tol) {
+                m.done = 1;
+            } else if (it >= itmax) {
+                m.status = AMG_ERR_NOT_CONVERGED;
+                m.done = 1;
+            }
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) *due = mask;
-    count_active(S, st, active, single);
+    count_active(S, st, active, due + 1, single);
 }
 
-__global__ void __launch_bounds__(kScalThreads) k_m_scal_replaced(Parts P, int S, const double* part_rr,
+__global__ void __launch_bounds__(kScalSys * 32) k_m_scal_replaced(Parts P, int S, const double* part_rr,
                                                                    const int* params, MultiState* st, int* active,
                                                                    unsigned* due, SolveState* single) {
     pdl_entry();
     if (*active == 0 || *due == 0) return;
-    SCAL_SHARED
-    sum_systems(P, S, part_rr, t0, sh);
-    const int itmax = params[0];
-    for (int s = threadIdx.x; s < S; s += blockDim.x) {
-        MultiState& m = st[s];
-        if (m.done || !m.replace_now) continue;
-        const double nr = sqrt(t0[s]);
-        m.nr = nr;
-        m.replace_now = 0;
-        if (isnan(nr) || isinf(nr)) {
-            m.status = AMG_ERR_NAN;
-            m.done = 1;
-        } else if (nr <= m.tol) {
-            m.done = 1;
-        } else if (m.iters >= itmax) {
-            m.status = AMG_ERR_NOT_CONVERGED;
-            m.done = 1;
+    SCAL_SYSTEM
+    if (s < S && !st[s].done && st[s].replace_now) {
+        const double rr = sum_system(P, s, part_rr, lane);
+        if (lane == 0) {
+            MultiState& m = st[s];
+            const double nr = sqrt(rr);
+            m.nr = nr;
+            m.replace_now = 0;
+            if (isnan(nr) || isinf(nr)) {
+                m.status = AMG_ERR_NAN;
+                m.done = 1;
+            } else if (nr <= m.tol) {
+                m.done = 1;
+            } else if (m.iters >= params[0]) {
+                m.status = AMG_ERR_NOT_CONVERGED;
+                m.done = 1;
+            }
         }
     }
-    if (threadIdx.x == 0) *due = 0;
-    count_active(S, st, active, single);
+    count_active(S, st, active, due + 1, single, due);
 }
 
-__global__ void __launch_bounds__(kScalThreads) k_m_scal_beta(Parts P, int S, const double* part_rz,
+__global__ void __launch_bounds__(kScalSys * 32) k_m_scal_beta(Parts P, int S, const double* part_rz,
                                                                const double* part_zq, int flexible, int first,
-                                                               MultiState* st, int* active, SolveState* single) {
+                                                               MultiState* st, int* active, unsigned* due,
+                                                               SolveState* single) {
     pdl_entry();
     if (*active == 0) return;
-    SCAL_SHARED
-    __shared__ double t1[kScalThreads];
+    SCAL_SYSTEM
     const bool flex = flexible && !first;
-    sum_systems(P, S, part_rz, t0, sh);
-    if (flex) sum_systems(P, S, part_zq, t1, sh);
-    for (int s = threadIdx.x; s < S; s += blockDim.x) {
-        MultiState& m = st[s];
-        if (m.done) continue;
-        const double rz = t0[s];
-        if (isnan(rz) || (flex && isnan(t1[s]))) {
-            m.status = AMG_ERR_NAN;
-            m.done = 1;
-            continue;
+    if (s < S && !st[s].done) {
+        const double rz = sum_system(P, s, part_rz, lane);
+        const double zq = flex ? sum_system(P, s, part_zq, lane) : 0.0;
+        if (lane == 0) {
+            MultiState& m = st[s];
+            if (isnan(rz) || isnan(zq)) {
+                m.status = AMG_ERR_NAN;
+                m.done = 1;
+            } else {
+                m.beta = first ? 0.0 : (flexible ? -zq / m.pq : rz / m.rho);
+                m.rho = rz;
+            }
         }
-        m.beta = first ? 0.0 : (flexible ? -t1[s] / m.pq : rz / m.rho);
-        m.rho = rz;
     }
-    count_active(S, st, active, single);
+    count_active(S, st, active, due + 1, single);
 }
 
 // dots[2 s], dots[2 s + 1] = the systems' sums (the final residual norms)
-__global__ void __launch_bounds__(kScalThreads) k_m_totals(Parts P, int S, const double* part0, const double* part1,
+__global__ void __launch_bounds__(kScalSys * 32) k_m_totals(Parts P, int S, const double* part0, const double* part1,
                                                             double* dots) {
     pdl_entry();
-    SCAL_SHARED
-    __shared__ double t1[kScalThreads];
-    sum_systems(P, S, part0, t0, sh);
-    sum_systems(P, S, part1, t1, sh);
-    for (int s = threadIdx.x; s < S; s += blockDim.x) {
-        dots[2 * s] = t0[s];
-        dots[2 * s + 1] = t1[s];
+    SCAL_SYSTEM
+    if (s >= S) return;
+    const double t0 = sum_system(P, s, part0, lane), t1 = sum_system(P, s, part1, lane);
+    if (lane == 0) {
+        dots[2 * s] = t0;
+        dots[2 * s + 1] = t1;
     }
 }
 
@@ -982,6 +967,7 @@ __global__ void k_deinterleave(int n, int R, int Rs, int64_t ld, const double* _
 }
 
 // ----------------------------------------------------------------- host side
+inline int scal_blocks(int S) { return (S + kScalSys - 1) / kScalSys; }
 inline int elem_blocks(int64_t count) { return (int)((count + 255) / 256 > 0 ? (count + 255) / 256 : 1); }
 
 template <typename A>
@@ -1266,12 +1252,12 @@ cudaError_t enqueue_multi_start(amg_hierarchy* h, cudaStream_t s) {
     MultiWork& w = *h->mw;
     Parts P;
     AMG_TRY(any_residual(h, w.r, true, true, false, &P, s));
-    launch_pdl(k_m_scal_init, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), h->rtol, h->itmax,
+    launch_pdl(k_m_scal_init, scal_blocks(w.S), kScalSys * 32, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), h->rtol, h->itmax,
                h->mixed ? h->o.resid_replace_every : 0, w.st, w.active, w.params, w.due, h->st);
     AMG_TRY(cudaGetLastError());
     AMG_TRY(any_vcycle(h, &P, s));
-    launch_pdl(k_m_scal_beta, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), h->o.flexible, 1, w.st,
-               w.active, h->st);
+    launch_pdl(k_m_scal_beta, scal_blocks(w.S), kScalSys * 32, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), h->o.flexible, 1, w.st,
+               w.active, w.due, h->st);
     any_pupdate(h, 1, s);
     return cudaGetLastError();
 }
@@ -1281,20 +1267,20 @@ cudaError_t enqueue_multi_iteration(amg_hierarchy* h, cudaStream_t s) {
     const int flex = h->o.flexible;
     Parts P;
     AMG_TRY(any_spmv_pq(h, &P, s));
-    launch_pdl(k_m_scal_alpha, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), flex, w.st, w.active,
-               h->st);
+    launch_pdl(k_m_scal_alpha, scal_blocks(w.S), kScalSys * 32, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), flex, w.st, w.active,
+               w.due, h->st);
     AMG_TRY(any_update(h, &P, s));
-    launch_pdl(k_m_scal_conv, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), h->mixed, w.params, w.st, w.active,
+    launch_pdl(k_m_scal_conv, scal_blocks(w.S), kScalSys * 32, 0, s, P, w.S, mslot(w, M_A), h->mixed, w.params, w.st, w.active,
                w.due, h->st);
     if (h->mixed) {  // FP64 true-residual replacement, when due
         AMG_TRY(any_residual(h, w.r, true, false, true, &P, s));
-        launch_pdl(k_m_scal_replaced, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), w.params, w.st, w.active, w.due,
+        launch_pdl(k_m_scal_replaced, scal_blocks(w.S), kScalSys * 32, 0, s, P, w.S, mslot(w, M_A), w.params, w.st, w.active, w.due,
                    h->st);
     }
     AMG_TRY(cudaGetLastError());
     AMG_TRY(any_vcycle(h, &P, s));
-    launch_pdl(k_m_scal_beta, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), flex, 0, w.st, w.active,
-               h->st);
+    launch_pdl(k_m_scal_beta, scal_blocks(w.S), kScalSys * 32, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), flex, 0, w.st, w.active,
+               w.due, h->st);
     any_pupdate(h, 0, s);
     return cudaGetLastError();
 }
@@ -1304,7 +1290,7 @@ cudaError_t enqueue_multi_final(amg_hierarchy* h, cudaStream_t s) {
     MultiWork& w = *h->mw;
     Parts P;
     AMG_TRY(any_residual(h, w.q, false, true, false, &P, s));
-    launch_pdl(k_m_totals, 1, kScalThreads, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), w.dots);
+    launch_pdl(k_m_totals, scal_blocks(w.S), kScalSys * 32, 0, s, P, w.S, mslot(w, M_A), mslot(w, M_B), w.dots);
     return cudaGetLastError();
 }
 
