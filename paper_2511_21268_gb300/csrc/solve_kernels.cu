@@ -561,12 +561,14 @@ int rows_per_warp(int n, int num_sms) {
 // a lane each where there are kShortFull rows per SM.  Measured in FP64: 2-D
 // p = 3 n = 101 (49 entries), q = K p 14.2 -> 5.2 us and the level-0 up sweep
 // 15.2 -> 5.6 us with 4 rows per warp instead of one; the coarse levels of 3-D
-// p = 2 n = 49 (75 to 95 entries) 95 -> 75 us per V-cycle; no gain at 226
-// entries, a loss at 1,200 (a Chebyshev step 18 -> 29 us).  FP32 keeps the
+// p = 2 n = 49 (75 to 95 entries) 95 -> 75 us per V-cycle; 17,401 rows of 154
+// entries (3-D p = 3 n = 65, level 2) 22 -> 15 us for residual and restriction,
+// 19 -> 15 us for the up sweep; no gain at 216 entries, a loss at 1,200 (a
+// Chebyshev step 18 -> 29 us).  FP32 keeps the
 // split of rows_per_warp in a single solve.  A batch in FP32 sums every row in
 // entry order (a lane per row): mixed-precision solutions of ill-conditioned
 // systems show in the ninth digit how their V-cycle rounds.
-constexpr int kShortRow = 128;
+constexpr int kShortRow = 180;
 constexpr int kShortFull = 512;
 int level_rows(const amg_hierarchy* h, const Level& L, bool batch) {
     const int64_t n = L.A.n, sms = h->num_sms;
