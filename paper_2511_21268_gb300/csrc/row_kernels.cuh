@@ -222,14 +222,7 @@ struct RunM {
     const V* __restrict__ v;
     template <typename A, typename X>
     __device__ __forceinline__ A partial(const X* __restrict__ x, int i, int lane) const {
-        return strided<32, A>(x, i, lane);
-    }
-    template <typename A, typename X>
-    __device__ __forceinline__ A sub(const X* __restrict__ x, int i, int q) const {
-        return strided<8, A>(x, i, q);
-    }
-    template <int S, typename A, typename X>
-    __device__ __forceinline__ A strided(const X* __restrict__ x, int i, int lane) const {
+        constexpr int S = 32;
         const int64_t b = __ldg(rp + i), e = __ldg(rp + i + 1);
         const uint32_t L = rlen[i];
         const uint32_t mg = kRunMagic[L];
