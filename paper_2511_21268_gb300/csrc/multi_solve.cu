@@ -37,7 +37,7 @@
 // mixed precision, us per pass before (a lane per right-hand side, every entry
 // a load of its own) and after: q = K p 102 -> 58, residual 106 -> 67, up
 // sweep 100 -> 59, a level below the first 33 and 19 -> 11 and 10, the dots and
-// scalars of an iteration 140 -> 31; 102.5 -> 50.9 ms a solve.
+// scalars of an iteration 140 -> 23; 102.5 -> 48.6 ms a solve.
 //
 // A batch's passes over level 0 (24 2-D systems, p 2..4, n 32..160, mixed
 // precision): 46, 40 and 35 us with a thread per row -> 27, 26 and 26 us with
@@ -413,6 +413,48 @@ __global__ void __launch_bounds__(kBlock, 2) k_m_resid(int n, int Rs, int lp, in
     });
 }
 
+// Residual and restriction of a level in one kernel, as k_resid_restrict: a
+// block takes `rows` coarse rows, a warp a member, and the residuals of the
+// members stay in shared memory.  Same sums in the same order.  For levels with
+// a warp for every row (at most 16 rows per SM): 16 right-hand sides, the two
+// small levels of 3-D p = 3 n = 32, 18.5 -> 12.3 us per V-cycle.  With the level
+// above them too, of 12 rows per warp, nothing more was gained (48.0 -> 48.2 ms a
+// solve).
+template <typename A, typename V>
+__global__ void __launch_bounds__(kBlock, 2) k_m_resid_restrict(
+    int nc, int rows, int Rs, int lp, MatM<V> mat, const A* __restrict__ f, const A* __restrict__ x,
+    const int32_t* __restrict__ mptr, const int32_t* __restrict__ midx, const double* __restrict__ pval, A* fc, A* xc,
+    const A* __restrict__ invdc, const int* active) {
+    pdl_entry();
+    if (*active == 0) return;
+    constexpr int kMembers = kWarpsPerBlock > kMaxMembers ? kWarpsPerBlock : kMaxMembers;
+    __shared__ A ts[kMembers][kMaxRs], ps[kMembers];
+    const Lanes L = lanes_of<A>(Rs, lp);
+    const int wid = threadIdx.x >> 5;
+    for (int J0 = blockIdx.x * rows; J0 < nc; J0 += gridDim.x * rows) {
+        const int J1 = min(J0 + rows, nc), m0 = mptr[J0], m1 = mptr[J1];
+        for (int m = m0 + wid; m < m1; m += kWarpsPerBlock) {
+            const int i = midx[m];
+            const A pi = (A)pval[i], fi = L.own ? f[(int64_t)i * Rs + L.c] : A(0);
+            const int64_t b = mat.rp[i];
+            A acc[kVec<A>];
+            row_dot<A, kBatch<A>>((int)(mat.rp[i + 1] - b), mat.v + b, mat.ci + b, x, Rs, L, acc);
+            const A s = reduce_columns(acc, L);
+            if (L.own && L.dup == 0) ts[m - m0][L.c] = fi - s;
+            if ((threadIdx.x & 31) == 0) ps[m - m0] = pi;
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < (J1 - J0) * Rs; t += kBlock) {
+            const int J = J0 + t / Rs, c = t % Rs;
+            A acc = A(0);
+            for (int m = mptr[J]; m < mptr[J + 1]; m++) acc = fma(ps[m - m0], ts[m - m0][c], acc);
+            fc[(int64_t)J * Rs + c] = acc;
+            if (xc) xc[(int64_t)J * Rs + c] = acc * invdc[J];
+        }
+        __syncthreads();
+    }
+}
+
 template <typename A>
 __global__ void k_m_restrict(int nc, int Rs, const int32_t* __restrict__ mptr, const int32_t* __restrict__ midx,
                              const double* __restrict__ pval, const A* __restrict__ rbuf, A* fc, A* xc,
@@ -431,13 +473,16 @@ __global__ void k_m_restrict(int nc, int Rs, const int32_t* __restrict__ mptr, c
     if (xc) xc[g] = acc * invdc[I];
 }
 
-// Coarsest level, e = A^-1 f per vector (FP64, a warp per row of the dense
-// inverse, one warp per block: the products spread over as many SMs' FP64
-// pipes as there are rows); prolongation into the finer level, or
-// (single-level hierarchy) z = e with the block partials of r.z and z.q.
-constexpr int kCoarseU = 8;  // entries of a lane group in flight
+// Coarsest level, e = A^-1 f per vector (FP64, a block of four warps per row of
+// the dense inverse: a warp issues one FP64 instruction in 64 cycles, and the
+// conversions of f are FP64 instructions too, so the row is split over the SM's
+// four pipes: 12.4 -> 7.5 us for 77 rows and 16 right-hand sides); prolongation
+// into the finer level, or (single-level hierarchy) z = e with the block
+// partials of r.z and z.q.
+constexpr int kCoarseU = 4;  // entries of a lane group in flight
+constexpr int kCoarseWarps = 4;
 template <typename FT, typename XT>
-__global__ void __launch_bounds__(32) k_m_coarse(int nd, int Rs, int lp, const double* __restrict__ Ainv,
+__global__ void __launch_bounds__(kCoarseWarps * 32) k_m_coarse(int nd, int Rs, int lp, const double* __restrict__ Ainv,
                                                   const FT* __restrict__ f, const int32_t* __restrict__ mptr,
                                                   const int32_t* __restrict__ midx,
                                                   const double* __restrict__ pvalf, XT* xf, double* z,
@@ -445,18 +490,18 @@ __global__ void __launch_bounds__(32) k_m_coarse(int nd, int Rs, int lp, const d
                                                   int flexible, const int* active) {
     pdl_entry();
     if (*active == 0) return;
-    __shared__ double sh[kMaxRs];
+    __shared__ double sh[kCoarseWarps * kMaxRs];
     const Lanes L = lanes_of<double>(Rs, lp);
-    const int G = 32 / lp;
+    const int G = 32 / lp, wid = threadIdx.x >> 5;
     double rz = 0.0, zq = 0.0;
-    SPMM_ROWS(I, nd) {
+    for (int I = blockIdx.x; I < nd; I += gridDim.x) {
         const double* __restrict__ row = Ainv + (int64_t)I * nd;
         double s2[2] = {0.0, 0.0};
-        for (int j0 = L.g; j0 < nd; j0 += kCoarseU * G) {
+        for (int j0 = L.g + wid * G; j0 - L.g < nd; j0 += kCoarseU * kCoarseWarps * G) {
             double a[kCoarseU], x0[kCoarseU], x1[kCoarseU];
 #pragma unroll
             for (int u = 0; u < kCoarseU; u++) {
-                const int j = j0 + u * G;
+                const int j = j0 + u * kCoarseWarps * G;
                 const bool in = j < nd;
                 const FT* fj = f + (int64_t)(in ? j : 0) * Rs + L.c0;
                 a[u] = in ? __ldg(row + j) : 0.0;
@@ -470,7 +515,13 @@ __global__ void __launch_bounds__(32) k_m_coarse(int nd, int Rs, int lp, const d
             }
         }
         __syncwarp();
-        const double s = reduce_columns(s2, L);
+        double s = reduce_columns(s2, L);
+        if (wid > 0 && L.own && L.dup == 0) sh[wid * kMaxRs + L.c] = s;
+        __syncthreads();
+        if (wid == 0 && L.own)
+            for (int w = 1; w < kCoarseWarps; w++) s += sh[w * kMaxRs + L.c];
+        __syncthreads();  // sh is free again
+        if (wid > 0) continue;
         if (z) {
             if (L.own && L.dup == 0) {
                 const int64_t e = (int64_t)I * Rs + L.c;
@@ -1066,7 +1117,7 @@ cudaError_t m_vcycle(amg_hierarchy* h, cudaStream_t s) {
     const int L = h->nlev, Rs = w.Rs, lp = lanes_per_entry<A>(Rs), flex = h->o.flexible;
     const int* act = w.active;
     if (L == 1) {
-        launch_pdl(k_m_coarse<double, A>, coarse_blocks(h), 32, 0, s, h->ndense, Rs,
+        launch_pdl(k_m_coarse<double, A>, coarse_blocks(h), kCoarseWarps * 32, 0, s, h->ndense, Rs,
                    lanes_per_entry<double>(Rs), h->Ainv, w.r, nullptr, nullptr, nullptr, nullptr, w.z, w.q,
                    mslot(w, M_A), mslot(w, M_B), flex, act);
         return cudaGetLastError();
@@ -1075,6 +1126,19 @@ cudaError_t m_vcycle(amg_hierarchy* h, cudaStream_t s) {
         Level& F = h->lev[l];
         Level& C = h->lev[l + 1];
         const int n = F.A.n, nb = spmm_blocks(h, n), T = rows_together<A>(h, n, Rs);
+        const bool coarsest = (l + 1 == L - 1);
+        A* xc = coarsest ? nullptr : Vw::x(w, l + 1);
+        if (l > 0 && n <= nb * kWarpsPerBlock) {  // a warp for every row
+            Vw::vals(F, l, [&](auto vp) {
+                using V = vt<decltype(vp)>;
+                const int rows = std::max(1, kWarpsPerBlock >> F.npass);
+                launch_pdl(k_m_resid_restrict<A, V>, std::max(1, std::min(2 * h->num_sms, (C.A.n + rows - 1) / rows)), kBlock, 0, s,
+                           C.A.n, rows, Rs, lp, mat_of(F, vp), static_cast<const A*>(Vw::f(w, l)),
+                           static_cast<const A*>(Vw::x(w, l)), F.mem_ptr, F.mem_idx, F.pval, Vw::f(w, l + 1), xc,
+                           Vw::invd(C), act);
+            });
+            continue;
+        }
         Vw::vals(F, l, [&](auto vp) {
             using V = vt<decltype(vp)>;
             if (l == 0)
@@ -1086,14 +1150,13 @@ cudaError_t m_vcycle(amg_hierarchy* h, cudaStream_t s) {
                 launch_pdl(k_m_resid<false, A, V, A>, nb, kBlock, 0, s, n, Rs, lp, T, mat_of(F, vp), Vw::f(w, l),
                            Vw::x(w, l), Vw::t(w, l), act);
         });
-        const bool coarsest = (l + 1 == L - 1);
         launch_pdl(k_m_restrict<A>, elem_blocks((int64_t)C.A.n * Rs), 256, 0, s, C.A.n, Rs, F.mem_ptr, F.mem_idx,
-                   F.pval, Vw::t(w, l), Vw::f(w, l + 1), coarsest ? nullptr : Vw::x(w, l + 1), Vw::invd(C), act);
+                   F.pval, Vw::t(w, l), Vw::f(w, l + 1), xc, Vw::invd(C), act);
     }
     {
         Level& F = h->lev[L - 2];
         Level& C = h->lev[L - 1];
-        launch_pdl(k_m_coarse<A, A>, coarse_blocks(h), 32, 0, s, C.A.n, Rs, lanes_per_entry<double>(Rs),
+        launch_pdl(k_m_coarse<A, A>, coarse_blocks(h), kCoarseWarps * 32, 0, s, C.A.n, Rs, lanes_per_entry<double>(Rs),
                    h->Ainv, Vw::f(w, L - 1), F.mem_ptr, F.mem_idx, F.pval, Vw::x(w, L - 2), nullptr, nullptr, nullptr,
                    nullptr, 0, act);
     }
