@@ -67,3 +67,29 @@ def test_small_solves_end_like_the_solve_by_launches(d, n, p):
             out = h.solve(gpu(F), **{"rtol": 1e-9, **kw})
             into += [out["status"], out["iters"]]
         assert got == ref or (kw == {} and got[0] == ref[0] == 0 and abs(got[1] - ref[1]) <= 1)
+
+
+def test_rows_that_do_not_fit_one_block():
+    """Few entries in all, but most of them in the rows of few coarse rows (a
+    dense block beside a chain): the launches solve it, on every call."""
+    m, c = 400, 2000
+    rp, ci, v = [0], [], []
+    for i in range(m):
+        ci.append(np.arange(m))
+        v.append(np.where(np.arange(m) == i, m + 0.5, -1.0))
+        rp.append(rp[-1] + m)
+    for i in range(c):
+        col = [j for j in (i - 1, i, i + 1) if 0 <= j < c]
+        ci.append(np.array(col) + m)
+        v.append(np.array([2.01 if j == i else -1.0 for j in col]))
+        rp.append(rp[-1] + len(col))
+    rp, ci, v = np.array(rp, np.int64), np.concatenate(ci).astype(np.int32), np.concatenate(v)
+    F = np.random.default_rng(2).normal(size=m + c)
+    H = A.Hierarchy(rp, ci, v)
+    assert H.num_levels > 1 and sum(H.level_nnz(l) for l in range(H.num_levels)) <= 200000
+    ref = O.Hierarchy(rp, ci, v).pcg(F, rtol=1e-9)
+    for _ in range(2):
+        out = H.solve(gpu(F), rtol=1e-9)
+        assert out["status"] == 0 and abs(out["iters"] - ref["iters"]) <= 1
+        if out["iters"] == ref["iters"]:
+            assert np.linalg.norm(out["u"].cpu().numpy() - ref["u"]) <= 1e-10 * np.linalg.norm(ref["u"])
