@@ -2,11 +2,11 @@
 // (arXiv 2511.21268, Sec. 3: CG with one V-cycle as preconditioner; FP64).
 //
 // A system of a few thousand rows is all latency: an iteration of the
-// stream-ordered solve is a dozen dependent launches of 2.5 to 4 us each (45 us
-// with its share of the fixed costs for the 1,024 rows of 2-D p = 2 n = 32, now
-// 29), with a few hundred nanoseconds of arithmetic in each.  Here the blocks of one cluster split the rows of every
-// level and keep them for the whole solve: a block owns a range of the
-// coarsest rows, and on every finer level the members of its rows.  What only
+// stream-ordered solve is a dozen dependent launches of 2.5 to 4 us each (41 us
+// with its share of the fixed costs for the 1,024 rows of 2-D p = 2 n = 32; here
+// 29), with a few hundred nanoseconds of arithmetic in each.  Here the blocks of
+// one cluster split the rows of every level and keep them for the whole solve: a
+// block owns a range of the coarsest rows, and on every finer level the members of its rows.  What only
 // the owner of a row touches -- matrix rows, diagonals, right-hand sides,
 // residuals, the CG vectors -- stays in the block's shared memory, restriction
 // and prolongation are local, and only the vectors that other blocks gather
@@ -564,14 +564,14 @@ cudaError_t cluster_config(amg_hierarchy* h, int C, cudaLaunchConfig_t& cfg, cud
 // the kernel knows), and a system for which it is the faster solve.  Measured
 // us per iteration of a whole solve to 1e-10, one cluster against the launches
 // of the iteration graph, by entries of the finest level:
-//   2-D: 27k (p = 3, n = 24) 21 / 33, 24k (p = 2, n = 32) 29 / 45, 76k (p = 3,
-//   n = 40) 31 / 44, 55k (p = 2, n = 48) 34 / 44, 99k (p = 2, n = 64) 45 / 53,
-//   155k (p = 2, n = 80) 56 / 56, 185k (p = 4, n = 48) 42 / 43, 196k (p = 3,
-//   n = 64) 52 / 50
-//   3-D: 39k (p = 2, n = 8) 22 / 51, 85k (p = 2, n = 10) 32 / 62, 133k (p = 3,
-//   n = 8) 31 / 78, 157k (p = 2, n = 12) 38 / 61
-// The line is where the 2-D systems break even.  16 blocks of 512 threads: 8
-// blocks took 1.05 times, 4 blocks 1.3 times as long, 256 threads the same.
+//   2-D: 27k (p = 3, n = 24) 21 / 32, 24k (p = 2, n = 32) 29 / 41, 76k (p = 3,
+//   n = 40) 31 / 39, 55k (p = 2, n = 48) 34 / 41, 99k (p = 2, n = 64) 43 / 48,
+//   185k (p = 4, n = 48) 42 / 40; 155k in 6,400 rows (p = 2, n = 80) do not fit
+//   3-D: 39k (p = 2, n = 8) 22 / 52, 85k (p = 2, n = 10) 31 / 61, 133k (p = 3,
+//   n = 8) 32 / 77, 157k (p = 2, n = 12) 38 / 60
+// The line (all levels) is where the 2-D systems break even.  16 blocks of 512
+// threads: 8 blocks took 1.05 times, 4 blocks 1.3 times as long, 256 threads the
+// same.
 int cluster_solve_blocks(amg_hierarchy* h) {
     if (h->mixed || h->prof || h->o.nu_pre != 1 || h->o.nu_post != 1 || h->o.cheb_degree > 0 ||
         h->o.coarse_solver != 0 || h->nlev < 2 || h->nlev > kClLevels)
