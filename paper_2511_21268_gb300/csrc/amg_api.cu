@@ -907,6 +907,28 @@ int join_caller(amg_hierarchy* h) {
 
 namespace amg {
 int join_caller_stream(amg_hierarchy* h) { return join_caller(h); }
+
+cudaError_t allow_smem_fn(const void* kernel, size_t bytes) {
+    // static shared memory of the kernels asked for (a property of the build)
+    static std::mutex mu;
+    static std::vector<std::pair<const void*, int>> sizes;
+    int dev = 0, optin = 0, fixed = -1;
+    AMG_TRY(cudaGetDevice(&dev));
+    AMG_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        for (const auto& k : sizes)
+            if (k.first == kernel) fixed = k.second;
+        if (fixed < 0) {
+            cudaFuncAttributes a;
+            AMG_TRY(cudaFuncGetAttributes(&a, kernel));
+            fixed = (int)a.sharedSizeBytes;
+            sizes.push_back({kernel, fixed});
+        }
+    }
+    if (bytes > (size_t)std::max(0, optin - fixed)) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - fixed);
+}
 int report_cuda(cudaError_t e, const char* what) { return cuda_fail(e, what); }
 }  // namespace amg
 

@@ -548,6 +548,18 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, siz
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+
+// Before a launch of `kernel` with `bytes` of dynamic shared memory, or the
+// setup of a hierarchy that will launch it: cudaErrorInvalidValue when they do
+// not fit beside the kernel's static shared memory.  A kernel's limit belongs
+// to the process, not to a hierarchy, so it is set to all that the device
+// allows and never to the size at hand: a smaller hierarchy would lower it
+// under a larger one, from another thread or before the larger one's solve.
+cudaError_t allow_smem_fn(const void* kernel, size_t bytes);
+template <typename K>
+inline cudaError_t allow_smem(K* kernel, size_t bytes) {
+    return allow_smem_fn(reinterpret_cast<const void*>(kernel), bytes);
+}
 }  // namespace amg
 
 #define AMG_TRY(expr)                          \

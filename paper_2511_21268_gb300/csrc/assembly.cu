@@ -853,9 +853,7 @@ extern "C" int amg_iga_assemble(const amg_iga_patch* P, int64_t* rowptr, int32_t
     if ((err = cudaGetLastError()) != cudaSuccess) return report_cuda(err, "amg_iga_assemble launch");
     // contractions: Q x 32 staging per block
     const size_t smo = (size_t)Q * kCtIn * sizeof(double);
-    if ((err = cudaFuncSetAttribute(k_iga_outer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smo)) !=
-        cudaSuccess)
-        return report_cuda(err, "amg_iga_assemble smem");
+    if ((err = allow_smem(k_iga_outer, smo)) != cudaSuccess) return report_cuda(err, "amg_iga_assemble smem");
     auto outer = [&](const double* X, int64_t O, int64_t IN, int Rr, const int* ss, const int* LL, const double* W,
                      int Lm, double* Y, int accumulate, int p1 = 0) {
         dim3 grid((unsigned)((IN + kCtIn - 1) / kCtIn), (unsigned)O);
@@ -935,7 +933,7 @@ extern "C" int amg_iga_assemble(const amg_iga_patch* P, int64_t* rowptr, int32_t
     const size_t smi = (size_t)G.ng * rows * (Q + 1) * sizeof(double);
     if (smi > (size_t)optin) return AMG_ERR_ARG;
     auto inner = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi);
+        cudaError_t e = allow_smem(kern, smi);
         if (e != cudaSuccess) return e;
         kern<<<AMG_GRID(nblk(RhR, rows)), kInThreads, smi, s>>>(d, G, rows, sp, Lp, rowptr, val);
         return cudaGetLastError();
@@ -944,8 +942,7 @@ extern "C" int amg_iga_assemble(const amg_iga_patch* P, int64_t* rowptr, int32_t
     if (err != cudaSuccess) return report_cuda(err, "amg_iga_assemble last contraction");
     if (F) {
         const size_t smf = (size_t)kInRows * (Q + 1) * sizeof(double);
-        if ((err = cudaFuncSetAttribute(k_iga_inner_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smf)) != cudaSuccess)
+        if ((err = allow_smem(k_iga_inner_dense, smf)) != cudaSuccess)
             return report_cuda(err, "amg_iga_assemble smem");
         k_iga_inner_dense<<<AMG_GRID(nblk((int64_t)m * m, kInRows)), 32 * kInRows, smf, s>>>(d, fb, s1, L1, W1, F);
     }

@@ -970,8 +970,7 @@ SellShape sell_shape(const SellLevel& S, int q) {
 
 template <int LM, typename V, typename Epi>
 bool sell_attr(uint32_t smem) {
-    return cudaFuncSetAttribute(k_sell<LM, V, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-           cudaSuccess;
+    return allow_smem(k_sell<LM, V, Epi>, smem) == cudaSuccess;
 }
 
 template <int LM>
@@ -1162,15 +1161,11 @@ int prepare_level(amg_hierarchy* h, SellLevel& S, int n, const int64_t* rp, cons
     const int cap = (int)std::min<int64_t>((int64_t)capr * LM, (optin - 1024 - 4 * (int64_t)capr) / es);
     const size_t fsm = (size_t)es * cap + 4 * (size_t)capr;
     if (fp64) {
-        if (cudaFuncSetAttribute(k_sell_fill<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm) !=
-            cudaSuccess)
-            return AMG_ERR_CUDA;
+        if (allow_smem(k_sell_fill<double>, fsm) != cudaSuccess) return AMG_ERR_CUDA;
         launch_pdl(k_sell_fill<double>, std::min(nsl, 65535), 256, fsm, h->s, n, nsl, G, LM, cap, capr, rp, rptr,
                    rlen, rst, slots, win, goff, rank_sel, v64, o64, nullptr, ors);
     } else {
-        if (cudaFuncSetAttribute(k_sell_fill<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm) !=
-            cudaSuccess)
-            return AMG_ERR_CUDA;
+        if (allow_smem(k_sell_fill<float>, fsm) != cudaSuccess) return AMG_ERR_CUDA;
         launch_pdl(k_sell_fill<float>, std::min(nsl, 65535), 256, fsm, h->s, n, nsl, G, LM, cap, capr, rp, rptr,
                    rlen, rst, slots, win, goff, rank_sel, v32, o32, o16, ors);
     }
@@ -1323,19 +1318,13 @@ int sell64_pick_warps(const SellLevel& S, int G) {
 }
 
 template <int LM>
-bool sell64_attrs_lm(int smem) {
-    return cudaFuncSetAttribute(k_sell64<LM, Epi64PQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(k_sell64<LM, Epi64Resid>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(k_sell64<LM, Epi64Up0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(k_sell64<LM, Epi64ChebStep>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(k_sell64<LM, Epi64ChebResid>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(k_sell64<LM, Epi64ChebPost0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-               cudaSuccess;
+bool sell64_attrs_lm(size_t smem) {
+    return allow_smem(k_sell64<LM, Epi64PQ>, smem) == cudaSuccess &&
+           allow_smem(k_sell64<LM, Epi64Resid>, smem) == cudaSuccess &&
+           allow_smem(k_sell64<LM, Epi64Up0>, smem) == cudaSuccess &&
+           allow_smem(k_sell64<LM, Epi64ChebStep>, smem) == cudaSuccess &&
+           allow_smem(k_sell64<LM, Epi64ChebResid>, smem) == cudaSuccess &&
+           allow_smem(k_sell64<LM, Epi64ChebPost0>, smem) == cudaSuccess;
 }
 
 }  // namespace
@@ -1357,7 +1346,7 @@ int sell64_prepare(amg_hierarchy* h, int* scratch) {
     const int rc = prepare_level(h, S, F0.A.n, F0.A.rowptr, F0.run_ptr, F0.run_len, F0.run_start, nullptr, false,
                                  scratch, optin, F0.A.val);
     if (rc != AMG_OK || !S.on) return rc;
-    const int smem = 2 * S.xbytes;
+    const size_t smem = 2 * (size_t)S.xbytes;
     bool attrs;
     switch (S.lm) {
         case 3: attrs = sell64_attrs_lm<3>(smem); break;

@@ -1858,7 +1858,7 @@ static size_t galerkin_smem(int cap) { return sizeof(uint64_t) * (size_t)cap; }
 cudaError_t launch_galerkin_count(const DevCSR& A, const int32_t* agg, const int32_t* mem0, const int32_t* mem1,
                                   int nc, int cap, int64_t* rowcnt, cudaStream_t s) {
     const size_t sm = galerkin_smem(cap);
-    if (sm > 48 * 1024) AMG_TRY(cudaFuncSetAttribute(k_galerkin_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) AMG_TRY(allow_smem(k_galerkin_count, sm));
     k_galerkin_count<<<AMG_GRID(blocks_for(nc, 1, 65536)), kBlock, sm, s>>>(nc, A.rowptr, A.col, agg, mem0, mem1, cap, rowcnt);
     return cudaGetLastError();
 }
@@ -1866,7 +1866,7 @@ cudaError_t launch_galerkin_count(const DevCSR& A, const int32_t* agg, const int
 cudaError_t launch_galerkin_fill(const DevCSR& A, const int32_t* agg, const double* pval, const int32_t* mem0,
                                  const int32_t* mem1, int cap, DevCSR& C, cudaStream_t s) {
     const size_t sm = galerkin_smem(cap);
-    if (sm > 48 * 1024) AMG_TRY(cudaFuncSetAttribute(k_galerkin_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) AMG_TRY(allow_smem(k_galerkin_fill, sm));
     k_galerkin_fill<<<AMG_GRID(blocks_for(C.n, 1, 65536)), kBlock, sm, s>>>(C.n, A.rowptr, A.col, A.val, agg, pval, mem0, mem1,
                                                                     cap, C.rowptr, C.col, C.val);
     return cudaGetLastError();
@@ -1890,7 +1890,7 @@ cudaError_t launch_galerkin_count_bitmap(const DevCSR& A, const int32_t* agg, co
                                          int nc, int cap, int words, int64_t* rowcnt, int* flag, cudaStream_t s) {
     const size_t sm = bitmap_smem(cap, words, false);
     if (sm > 48 * 1024)
-        AMG_TRY(cudaFuncSetAttribute(k_galerkin_bitmap<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        AMG_TRY(allow_smem(k_galerkin_bitmap<false>, sm));
     k_galerkin_bitmap<false><<<AMG_GRID(blocks_for(nc, 1, 65536)), kGalerkinBlock, sm, s>>>(
         nc, A.rowptr, A.col, A.val, agg, nullptr, mem0, mem1, cap, words, rowcnt, nullptr, nullptr, nullptr, flag);
     return cudaGetLastError();
@@ -1900,7 +1900,7 @@ cudaError_t launch_galerkin_fill_bitmap(const DevCSR& A, const int32_t* agg, con
                                         const int32_t* mem1, int cap, int words, DevCSR& C, int* flag, cudaStream_t s) {
     const size_t sm = bitmap_smem(cap, words, true);
     if (sm > 48 * 1024)
-        AMG_TRY(cudaFuncSetAttribute(k_galerkin_bitmap<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        AMG_TRY(allow_smem(k_galerkin_bitmap<true>, sm));
     k_galerkin_bitmap<true><<<AMG_GRID(blocks_for(C.n, 1, 65536)), kGalerkinBlock, sm, s>>>(
         C.n, A.rowptr, A.col, A.val, agg, pval, mem0, mem1, cap, words, nullptr, C.rowptr, C.col, C.val, flag);
     return cudaGetLastError();
@@ -1939,7 +1939,7 @@ cudaError_t launch_galerkin_warp_count(const DevCSR& A, const int32_t* agg, cons
                                        int nc, int cmax, int64_t* rowcnt, int* stats, int* flag, cudaStream_t s) {
     const size_t sm = galerkin_warp_bytes(cmax, kGalCountWords, 0, false);
     if (sm > 48 * 1024)
-        AMG_TRY(cudaFuncSetAttribute(k_galerkin_warp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        AMG_TRY(allow_smem(k_galerkin_warp<false>, sm));
     // rows in flight are bounded by shared memory: ask for the largest carveout
     AMG_TRY(cudaFuncSetAttribute(k_galerkin_warp<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared));
@@ -1956,7 +1956,7 @@ cudaError_t launch_galerkin_warp_fill(const DevCSR& A, const int32_t* agg, const
                                       DevCSR& C, int* flag, cudaStream_t s) {
     const size_t sm = galerkin_warp_bytes(cmax, words, umax, true);
     if (sm > 48 * 1024)
-        AMG_TRY(cudaFuncSetAttribute(k_galerkin_warp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        AMG_TRY(allow_smem(k_galerkin_warp<true>, sm));
     AMG_TRY(cudaFuncSetAttribute(k_galerkin_warp<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared));
     int res = 0;
@@ -2022,15 +2022,13 @@ __global__ void k_keep_factor(int n, const double* __restrict__ D, double* L) {
 // the second n^2 (work space of the inverse before).
 cudaError_t launch_dense_spd_inverse(int n, double* D, double* Ainv, int* flag, cudaStream_t s) {
     bool done = false;
-    int optin = 0, dev = 0;
-    AMG_TRY(cudaGetDevice(&dev));
-    AMG_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     // one cluster where its shared memory holds the rows (16 blocks where the
     // device schedules such a cluster: n up to about 640; else 8: 450)
     for (int C = kCholMaxC; C >= 8 && !done; C >>= 1) {
         const size_t sm = sizeof(double) * (size_t)n * (4 + (n + C - 1) / C);
-        if (sm > (size_t)optin) continue;
-        AMG_TRY(cudaFuncSetAttribute(k_cholesky_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        const cudaError_t fits = allow_smem(k_cholesky_cluster, sm);
+        if (fits == cudaErrorInvalidValue) continue;
+        AMG_TRY(fits);
         if (C > 8 && cudaFuncSetAttribute(k_cholesky_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
                          cudaSuccess) {
             cudaGetLastError();
@@ -2059,13 +2057,14 @@ cudaError_t launch_dense_spd_inverse(int n, double* D, double* Ainv, int* flag, 
     }
     if (!done) k_cholesky<<<AMG_GRID(1), 1024, 0, s>>>(n, D, flag);
     const size_t smi = sizeof(double) * (2 + (size_t)n + (size_t)n * (n + 1) / 2);
-    if (n <= kInvThreads * kInvRegs && smi <= (size_t)optin) {
-        AMG_TRY(cudaFuncSetAttribute(k_chol_inverse_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi));
+    cudaError_t fits = cudaErrorInvalidValue;
+    if (n <= kInvThreads * kInvRegs) fits = allow_smem(k_chol_inverse_smem, smi);
+    if (fits != cudaErrorInvalidValue) {
+        AMG_TRY(fits);
         k_chol_inverse_smem<<<AMG_GRID(n), kInvThreads, smi, s>>>(n, D, Ainv);
     } else {
         const size_t sm = sizeof(double) * (size_t)n;  // the diagonal's reciprocals (n <= 8192: 64 KB)
-        if (sm > 48 * 1024)
-            AMG_TRY(cudaFuncSetAttribute(k_chol_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        if (sm > 48 * 1024) AMG_TRY(allow_smem(k_chol_inverse, sm));
         k_chol_inverse<<<AMG_GRID(blocks_for(n, kWarpsPerBlock, 4096)), kBlock, sm, s>>>(n, D, Ainv,
                                                                                         Ainv + (int64_t)n * n);
     }

@@ -679,9 +679,7 @@ static int spgemm(amg_hierarchy* h, int nA, const int64_t* arp, const int32_t* a
     // shared memory of the block-per-row kernel beyond bits/pre/acc: staged
     // A entries (8 + 8 + 4 bytes each) and the reduction scratch
     const size_t blk_tail = (size_t)20 * bt + 4 * (2 * (bt / 32) + 1) + 16;
-    auto cfg = [&](auto kern, size_t bytes) {
-        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    };
+    auto cfg = [&](auto kern, size_t bytes) { return allow_smem(kern, bytes); };
     auto blocks_blk = [&]() { return (int)std::max<int64_t>(1, std::min<int64_t>(nA, (int64_t)1 << 20)); };
     // the counting pass's row bitmaps, kept for the later pass when they fit the budget
     uint32_t* gbits = nullptr;

@@ -369,7 +369,7 @@ __global__ void k_block_window(int n, int S, int G, const int64_t* __restrict__ 
 template <int RPW, typename V, typename Epi>
 bool set_attrs(uint32_t smem) {
     auto fn = k_stream<RPW, V, Epi>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
+    if (allow_smem(fn, smem) != cudaSuccess) return false;
     return cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
 }
 
