@@ -604,14 +604,15 @@ int build(amg_hierarchy* h, const amg_csr* K) {
         RC(dalloc(h, &F.dl1, n));
         RC(dalloc(h, &F.invd, n));
         if (l == 0) {
-            CK(cudaMemsetAsync(h->flag, 0, 16 * sizeof(int), s));  // also clears the deferred error words
-            CK(launch_l1diag(F.A, F.kii, F.dl1, F.invd, h->flag, s));
+            // also clears the deferred error words and the row lengths
+            CK(cudaMemsetAsync(h->flag, 0, (kFlagRows + AMG_MAX_LEVELS) * sizeof(int), s));
+            CK(launch_l1diag(F.A, F.kii, F.dl1, F.invd, h->flag, h->flag + kFlagRows, s));
             RC(read_flag(h, &bad));
             if (bad) return AMG_ERR_NOT_SPD;
             // the finest level will have a smoother: start its network now
             if (h->o.mpnn_weights && n > h->o.coarse_max && h->o.max_levels > 1) RC(mpnn_setup_fork(h));
         } else {  // coarse levels: checked once after the loop (flag[4])
-            CK(launch_l1diag(F.A, F.kii, F.dl1, F.invd, h->flag + 4, s));
+            CK(launch_l1diag(F.A, F.kii, F.dl1, F.invd, h->flag + 4, h->flag + kFlagRows + l, s));
         }
         h->nlev = l + 1;
         if (n <= h->o.coarse_max || l + 1 >= h->o.max_levels) break;
@@ -690,8 +691,9 @@ int build(amg_hierarchy* h, const amg_csr* K) {
         C.w = cw;
     }
     // deferred checks of the coarse levels: Galerkin structure, positive diagonals
-    CK(cudaMemcpyAsync(h->flag_host, h->flag, 8 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(h->flag_host, h->flag, (kFlagRows + h->nlev) * sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    for (int l = 0; l < h->nlev; l++) h->lev[l].maxrow = h->flag_host[kFlagRows + l];
     if (h->flag_host[3]) return AMG_ERR_ARG;  // structurally unsymmetric input
     if (h->flag_host[4]) return AMG_ERR_NOT_SPD;
     // coarsest level: dense inverse
@@ -1043,7 +1045,7 @@ static int create_hierarchy(const amg_opts* opts, void* cuda_stream, amg_hierarc
         return rc;
     }
     rc = join_caller(h);
-    if (rc == AMG_OK) rc = dalloc(h, &h->flag, 16);
+    if (rc == AMG_OK) rc = dalloc(h, &h->flag, kFlagRows + AMG_MAX_LEVELS);
     if (rc != AMG_OK) {
         destroy(h);
         return rc;

@@ -131,7 +131,7 @@ struct Level {
     // runs interleaved (entry o of run r at rowptr[i] + o R + r)
     __nv_bfloat16* val16t = nullptr;
     float* val32t = nullptr;
-    int maxrow = 0;
+    int maxrow = 0;  // entries of the longest row
     // run-encoded columns (level 0, when every row is a sequence of equal
     // runs of consecutive columns): row i has run_ptr[i+1] - run_ptr[i] runs
     // of run_len[i] entries; run r starts at column run_start[r] and at entry
@@ -189,7 +189,7 @@ struct amg_hierarchy {
     std::vector<void*> allocs;   // device allocations owned by the hierarchy
     amg::SolveState* st = nullptr;
     amg::SolveState* st_host = nullptr;  // pinned mirror
-    int* flag = nullptr;                 // device scratch flag / counter
+    int* flag = nullptr;                 // device scratch flags / counters, then each level's longest row
     int* flag_host = nullptr;            // pinned mirror
     double* hist = nullptr;              // residual history (device)
     int hist_cap = 0;
@@ -254,7 +254,9 @@ namespace amg {
 // ----------------------------------------------------------------- launch wrappers
 // setup_kernels.cu
 cudaError_t launch_validate_csr(const DevCSR& A, int* flag, cudaStream_t s);
-cudaError_t launch_l1diag(const DevCSR& A, double* kii, double* dl1, double* invd, int* flag, cudaStream_t s);
+// also the entries of A's longest row, if more, into *longest
+cudaError_t launch_l1diag(const DevCSR& A, double* kii, double* dl1, double* invd, int* flag, int* longest,
+                          cudaStream_t s);
 cudaError_t launch_diag(const DevCSR& A, double* kii, cudaStream_t s);
 cudaError_t launch_testvec_init(int n, int kind, uint64_t seed, double* w, cudaStream_t s);
 cudaError_t launch_testvec_sweep(const DevCSR& A, const double* dl1, const double* w, double* wout, cudaStream_t s);
@@ -401,6 +403,7 @@ cudaError_t launch_run_rows(const DevCSR& A, int32_t* runcnt, uint8_t* runlen, i
 cudaError_t launch_run_fill(const DevCSR& A, const int32_t* run_ptr, const uint8_t* runlen, int32_t* run_start,
                             cudaStream_t s);
 int rows_per_warp(int n, int num_sms);
+constexpr int kFlagRows = 16;  // position of level 0's longest row in the flags
 int level_rows(const amg_hierarchy* h, const Level& L, bool batch);
 int row_blocks(int n, int rpw);
 int vec_blocks(int n, int num_sms);

@@ -228,13 +228,14 @@ inline bool fold_narrow(int n, int num_sms) { return (int64_t)(n + 31) / 32 >= 3
 template <int CW>
 __global__ void __launch_bounds__(kBlock, 3) k_l1diag(int n, const int64_t* __restrict__ rp,
                                                     const int32_t* __restrict__ ci, const double* __restrict__ v,
-                                                    double* kii, double* dl1, double* invd, int* flag) {
+                                                    double* kii, double* dl1, double* invd, int* flag, int* longest) {
     __shared__ double tiles[kWarpsPerBlock][32][CW + 1];
     __shared__ double diags[kWarpsPerBlock][32];  // the rows' diagonal entries (0 when a row has none)
     double(*tile)[CW + 1] = tiles[threadIdx.x >> 5];
     double* dg = diags[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    int len = 0;
     for (int row0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; row0 < n; row0 += nwarps * 32) {
         dg[lane] = 0.0;
         __syncwarp();
@@ -255,8 +256,12 @@ __global__ void __launch_bounds__(kBlock, 3) k_l1diag(int n, const int64_t* __re
             const double dl = __dadd_rn(d, s);
             dl1[i] = dl;
             if (invd) invd[i] = __ddiv_rn(1.0, dl);
+            len = max(len, (int)(rp[i + 1] - rp[i]));
         }
     }
+    __syncwarp();
+    len = __reduce_max_sync(0xffffffffu, len);
+    if (lane == 0 && len > __ldcg(longest)) atomicMax(longest, len);
 }
 
 __global__ void k_diag(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
@@ -1737,7 +1742,8 @@ cudaError_t launch_validate_csr(const DevCSR& A, int* flag, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_l1diag(const DevCSR& A, double* kii, double* dl1, double* invd, int* flag, cudaStream_t s) {
+cudaError_t launch_l1diag(const DevCSR& A, double* kii, double* dl1, double* invd, int* flag, int* longest,
+                          cudaStream_t s) {
     if (A.n == 0) return cudaSuccess;
     AMG_TRY(cudaMemsetAsync(kii, 0, sizeof(double) * A.n, s));
     int dev = 0, sms = 148;
@@ -1745,10 +1751,10 @@ cudaError_t launch_l1diag(const DevCSR& A, double* kii, double* dl1, double* inv
     AMG_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (fold_narrow(A.n, sms))
         k_l1diag<8><<<AMG_GRID(blocks_for(A.n, kBlock, 4096)), kBlock, 0, s>>>(A.n, A.rowptr, A.col, A.val, kii, dl1,
-                                                                              invd, flag);
+                                                                              invd, flag, longest);
     else
         k_l1diag<32><<<AMG_GRID(blocks_for(A.n, kBlock, 4096)), kBlock, 0, s>>>(A.n, A.rowptr, A.col, A.val, kii, dl1,
-                                                                               invd, flag);
+                                                                               invd, flag, longest);
     return cudaGetLastError();
 }
 

@@ -558,25 +558,35 @@ int rows_per_warp(int n, int num_sms) {
 // or a batch.  FP64 sums may be split over lanes in any way (the difference is
 // their rounding): short rows (at most kShortRow entries on average) take 8
 // lanes each, 4 rows per warp, where there is a warp's work for every SM, and
-// a lane each where there are kShortFull rows per SM.  Measured in FP64: 2-D
+// a lane each where there are kShortFull rows per SM, as long as no row is much
+// longer than that: the warps of the longest rows are a kernel's end.  Measured in FP64: 2-D
 // p = 3 n = 101 (49 entries), q = K p 14.2 -> 5.2 us and the level-0 up sweep
 // 15.2 -> 5.6 us with 4 rows per warp instead of one; the coarse levels of 3-D
 // p = 2 n = 49 (75 to 95 entries) 95 -> 75 us per V-cycle; 17,401 rows of 154
 // entries (3-D p = 3 n = 65, level 2) 22 -> 15 us for residual and restriction,
 // 19 -> 15 us for the up sweep; no gain at 216 entries, a loss at 1,200 (a
-// Chebyshev step 18 -> 29 us).  FP32 keeps the
+// Chebyshev step 18 -> 29 us).  A few long rows among short ones, us per V-cycle
+// with a lane each / 8 lanes / the split of rows_per_warp: 90,000 rows of 5
+// entries, the longest 105 entries 135 / 144 / 177, 155: 157 / 155 / 183, 305:
+// 203 / 171 / 181, 405: 240 / 187 / 185, 2,000: 705 / 347 / 219 (of 48 entries,
+// the longest 149: 154 / 141 / 181, 349: 213 / 162 / 182); 10,000 rows of 5,
+// the longest 205: - / 89 / 92, 302: - / 96 / 93, 1,833: - / 184 / 115; 13,824 of
+// 107, the longest 275: - / 99 / 100, 421: - / 108 / 105: kLaneLongest and
+// kShortLongest lie where they meet.  FP32 keeps the
 // split of rows_per_warp in a single solve.  A batch in FP32 sums every row in
 // entry order (a lane per row): mixed-precision solutions of ill-conditioned
 // systems show in the ninth digit how their V-cycle rounds.
 constexpr int kShortRow = 180;
 constexpr int kShortFull = 512;
+constexpr int kLaneLongest = 128;   // entries of the longest row, at most, with a lane per row
+constexpr int kShortLongest = 320;  // and with 8 lanes
 int level_rows(const amg_hierarchy* h, const Level& L, bool batch) {
     const int64_t n = L.A.n, sms = h->num_sms;
     const int plain = rows_per_warp(L.A.n, h->num_sms);
     if (n == 0) return plain;
     if (h->mixed) return batch ? 32 : plain;
-    if (L.A.nnz > kShortRow * n || n < sms * 4) return plain;
-    return n >= sms * kShortFull ? 32 : 4;
+    if (L.A.nnz > kShortRow * n || L.maxrow > kShortLongest || n < sms * 4) return plain;
+    return n >= sms * kShortFull && L.maxrow <= kLaneLongest ? 32 : 4;
 }
 
 int row_blocks(int n, int rpw) {
