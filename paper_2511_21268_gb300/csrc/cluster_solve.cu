@@ -33,6 +33,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "amg_internal.cuh"
 
 namespace amg {
@@ -47,6 +49,9 @@ constexpr int kClLevels = 8;  // levels, at most
 constexpr int kClIters = 64;  // iterations of one launch
 constexpr int kClStatic = 4096;  // static shared memory and slack
 constexpr int64_t kClusterNnz = 200000;  // entries of all levels, at most
+constexpr int64_t kClusterRows = 6000;   // rows of all levels and what counts as rows, at most:
+constexpr int64_t kClusterDense = 100;   //   products of the coarsest inverse per row
+constexpr int64_t kClusterLongest = 9;   //   rows per entry of the longest row
 
 struct ClLevel {
     int n;
@@ -560,30 +565,49 @@ cudaError_t cluster_config(amg_hierarchy* h, int C, cudaLaunchConfig_t& cfg, cud
 
 // Blocks of the cluster solve, 0 where it does not apply: FP64, one l1-Jacobi
 // sweep before and after, tentative prolongators, the dense coarsest solve,
-// no kernel timing, rows that fit the blocks' shared memory (an estimate here;
-// the kernel knows), and a system for which it is the faster solve.  Measured
-// us per iteration of a whole solve to 1e-10, one cluster against the launches
-// of the iteration graph, by entries of the finest level:
+// no kernel timing, and a system for which it is the faster solve.  (Whether the
+// rows fit the blocks' shared memory the kernel finds out.)  What the blocks have
+// to do per iteration is bounded by three lines.
+// Entries of all levels, at most kClusterNnz: measured us per iteration of a whole
+// solve to 1e-10, one cluster against the launches of the iteration graph, by
+// entries of the finest level:
 //   2-D: 27k (p = 3, n = 24) 21 / 32, 24k (p = 2, n = 32) 29 / 41, 76k (p = 3,
 //   n = 40) 31 / 39, 55k (p = 2, n = 48) 34 / 41, 99k (p = 2, n = 64) 43 / 48,
 //   185k (p = 4, n = 48) 42 / 40; 155k in 6,400 rows (p = 2, n = 80) do not fit
 //   3-D: 39k (p = 2, n = 8) 22 / 52, 85k (p = 2, n = 10) 31 / 61, 133k (p = 3,
 //   n = 8) 32 / 77, 157k (p = 2, n = 12) 38 / 60
-// The line (all levels) is where the 2-D systems break even.  16 blocks of 512
-// threads: 8 blocks took 1.05 times, 4 blocks 1.3 times as long, 256 threads the
-// same.
+// The line is where the 2-D systems break even (3-D systems, with fewer rows, would
+// gain some way above it).
+// Rows of all levels, plus the n^2 products of the coarsest inverse by
+// kClusterDense, plus the longest row's entries by kClusterLongest, at most
+// kClusterRows.  A row costs its share of the vector work and the reductions on 16
+// SMs, the dense products run on 16 SMs that the launches spread over all, and the
+// blocks of a phase wait for the longest row, which has 4 lanes.  Us per iteration,
+// cluster / launches:
+//   few entries per row (5,769 rows of all levels at n = 64): 5-point 32^2
+//   23 / 34, 64^2 40 / 42, 80^2 50 / 45, 100^2 73 / 54; 7-point 16^3 41 / 42, 20^3
+//   58 / 45; 3-point 2,000 32 / 39, 4,000 40 / 40, 6,000 55 / 50, 12,000 80 / 55
+//   coarsest rows: 5-point 64^2 with 108 40 / 42, 356 38 / 36, 1,209 63 / 32;
+//   2-D p = 2 n = 48 with 170 29 / 35, 619 34 / 30; 3-point 6,000 with 1,908 116 / 38
+//   longest row: 5-point 50^2 (3,510 rows) with 153 entries 50 / 56, 293 62 / 61,
+//   380 96 / 72, 695 101 / 81; 30^2 (1,240) with 440 41 / 52, 527 57 / 58; 2-D p = 2
+//   n = 32 (1,370) with 281 42 / 46, 480 55 / 55, 576 63 / 58
+// 16 blocks of 512 threads: 8 blocks took 1.05 times, 4 blocks 1.3 times as long, 256
+// threads the same.
 int cluster_solve_blocks(amg_hierarchy* h) {
     if (h->mixed || h->prof || h->o.nu_pre != 1 || h->o.nu_post != 1 || h->o.cheb_degree > 0 ||
         h->o.coarse_solver != 0 || h->nlev < 2 || h->nlev > kClLevels)
         return 0;
     if (h->cluster_blocks >= 0) return h->cluster_blocks;
     h->cluster_blocks = 0;
-    int64_t nnz = 0;
+    int64_t nnz = 0, rows = (int64_t)h->ndense * h->ndense / kClusterDense, longest = 0;
     for (int l = 0; l < h->nlev; l++) {
         if (h->lev[l].smoothed) return 0;
         nnz += h->lev[l].A.nnz;
+        rows += h->lev[l].A.n;
+        if (l + 1 < h->nlev) longest = std::max<int64_t>(longest, h->lev[l].maxrow);
     }
-    if (nnz > kClusterNnz) return 0;
+    if (nnz > kClusterNnz || rows + kClusterLongest * longest > kClusterRows) return 0;
     int dev = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
