@@ -170,8 +170,9 @@ typedef struct {
     int32_t staged_window_bytes; /* largest per-block vector window of the staged passes */
     int32_t staged_level1; /* 1: level 1 also runs sliced staged passes (plain CSR, FP32 values) */
     double graph_build_ms; /* host time capturing and instantiating the iteration graph in the last
-                              solve (0 when the hierarchy's graph was reused, and where a small
-                              system's solve is one kernel and has no graph) */
+                              solve (0 when the hierarchy's graph was reused, and where there is
+                              none: a small system's solve by one kernel, a system that was
+                              solved already) */
     int32_t smoothed[AMG_MAX_LEVELS]; /* 1 where the level's prolongator is smoothed */
     int64_t p_nnz[AMG_MAX_LEVELS];    /* stored entries of each level's prolongator */
     int32_t sell64_warps;  /* warps per block of the FP64 sliced passes (0 when not in use) */

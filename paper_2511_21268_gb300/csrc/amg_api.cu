@@ -956,6 +956,32 @@ int check_opts(const amg_opts& o) {
     return AMG_OK;
 }
 
+// The iterations of a first solve that run by launches, behind a copy of the
+// start phase's state to the host.  Once that has arrived and solved() says so
+// (F = 0, a converged guess: no iteration runs), *go_on becomes false: neither
+// more of them nor the graph are needed.  The host never waits with less than
+// eight iterations enqueued (a wait behind the first: 2-D p = 3 n = 101 setup and
+// solve 4.65 -> 4.68 ms).
+template <typename Solved>
+int first_iterations(amg_hierarchy* h, cudaError_t (*iteration)(amg_hierarchy*, cudaStream_t), Solved&& solved,
+                     bool* go_on) {
+    cudaError_t arrived = cudaErrorNotReady;
+    CK(cudaEventRecord(h->evs, h->s));
+    for (int k = 0; k < kGraphIters && *go_on; k++) {
+        CK(iteration(h, h->s));
+        if (arrived == cudaSuccess) continue;
+        arrived = cudaEventQuery(h->evs);
+        if (arrived == cudaErrorNotReady) (void)cudaGetLastError();  // not a failure
+        else CK(arrived);
+        if (arrived == cudaSuccess) *go_on = !solved();
+    }
+    if (arrived != cudaSuccess) {
+        CK(cudaEventSynchronize(h->evs));
+        *go_on = !solved();
+    }
+    return AMG_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1179,12 +1205,15 @@ static int run_solve(amg_hierarchy* h, int32_t* iters) {
         }
     }
     if (!cluster) CK(enqueue_pcg_start(h, s));
-    if (!cluster && !h->graph) {
+    bool build_graph = !cluster && !h->graph;
+    if (build_graph && !h->prof) {
         // The first iterations run by launches, and the graph (0.2 to 0.5 ms of
         // host time) is built meanwhile: 2-D p = 3 n = 101 setup and solve 4.83 ->
         // 4.66 ms, 3-D p = 2 n = 47 mixed 10.04 -> 9.93 ms.
-        if (!h->prof)
-            for (int k = 0; k < kGraphIters; k++) CK(enqueue_pcg_iteration(h, s));
+        CK(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
+        RC(first_iterations(h, enqueue_pcg_iteration, [&] { return h->st_host->done != 0; }, &build_graph));
+    }
+    if (build_graph) {
         const auto tb0 = std::chrono::steady_clock::now();
         cudaGraph_t g;
         const long long before = amg::g_launches.load();
@@ -1361,8 +1390,14 @@ static int run_multi(amg_hierarchy* h, int32_t* iters, double* relres, int32_t* 
     cudaStream_t s = h->s;
     CK(cudaEventRecord(h->ev0, s));
     CK(enqueue_multi_start(h, s));
-    if (!w.graph) {
-        for (int k = 0; k < kGraphIters; k++) CK(enqueue_multi_iteration(h, s));  // as in run_solve
+    bool build_graph = !w.graph;
+    h->info.graph_build_ms = 0.0;
+    if (build_graph) {  // as in run_solve
+        CK(cudaMemcpyAsync(h->flag_host, w.active, sizeof(int), cudaMemcpyDeviceToHost, s));
+        RC(first_iterations(h, enqueue_multi_iteration, [&] { return *h->flag_host == 0; }, &build_graph));
+    }
+    if (build_graph) {
+        const auto tb0 = std::chrono::steady_clock::now();
         cudaGraph_t g;
         const long long before = amg::g_launches.load();
         CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -1379,6 +1414,8 @@ static int run_multi(amg_hierarchy* h, int32_t* iters, double* relres, int32_t* 
             w.graph = nullptr;
             return cuda_fail(e, "cudaGraphInstantiate");
         }
+        h->info.graph_build_ms =
+            std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tb0).count();
     }
     const int max_launches = h->itmax / kGraphIters + 2;
     for (int k = 0; k <= max_launches + 1; k++) {
