@@ -1349,7 +1349,7 @@ static int ensure_multi(amg_hierarchy* h, int R, int S, const int32_t* seg) {
         w->F = h->F;
         w->p32 = h->p32;
     } else {
-        w->Rs = (R + 3) & ~3;
+        w->Rs = h->mixed ? (R + 3) & ~3 : (R + 1) & ~1;  // 16 bytes per lane
         const size_t E = (size_t)h->lev[0].A.n * w->Rs;
         for (double** v : {&w->x, &w->r, &w->p, &w->q, &w->z, &w->F}) {
             RC(walloc(h, *w, v, E));

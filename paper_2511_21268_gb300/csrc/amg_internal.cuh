@@ -49,7 +49,8 @@ struct MultiState {
 };
 
 // Workspace of a multi-system solve.  Several right-hand sides: vectors
-// interleaved [N][Rs], Rs = R rounded up to a multiple of 4.  Batch: the
+// interleaved [N][Rs], Rs = R rounded up to 16 bytes of the V-cycle's
+// precision: a multiple of 4 in FP32, of 2 in FP64.  Batch: the
 // hierarchy's own vectors, and the systems' rows in tiles.
 struct MultiWork {
     int R = 0, Rs = 0, S = 0;

@@ -3,7 +3,8 @@
 // the batching is this library's design).
 //
 //   * R right-hand sides of one matrix (k_m_*): vectors interleaved as
-//     [N][Rs], Rs = R rounded up to a multiple of 4, the padding columns
+//     [N][Rs], Rs = R rounded up to a multiple of 4 (mixed precision) or 2
+//     (FP64), so that a row is whole 16-byte pieces; the padding columns
 //     zero; a matrix pass reads each matrix entry once for all R vectors
 //     (SpMM).  System s = right-hand side s.
 //   * a batch of independent matrices assembled block-diagonally into one
@@ -38,6 +39,13 @@
 // a load of its own) and after: q = K p 102 -> 58, residual 106 -> 67, up
 // sweep 100 -> 59, a level below the first 33 and 19 -> 11 and 10, the dots and
 // scalars of an iteration 140 -> 23; 102.5 -> 48.6 ms a solve.
+//
+// Few right-hand sides in FP64, us per iteration of a solve with a lane per
+// right-hand side / rows of four columns / of two (now, 1 or 2 right-hand sides):
+// 3-D p = 3 n = 24 400 / 220 / 168, 3-D p = 2 n = 40 490 / 442 / 343, 2-D p = 3 n =
+// 101 144 / 100 / 102; workspace of one, bytes per row (4 M rows of 5 entries): 84 /
+// 294 / 143.  In mixed precision one to three columns are carried as four: 385 to
+// 427 -> 120 us, 436 to 461 -> 222 and 160 -> 94 on the same systems.
 //
 // A batch's passes over level 0 (24 2-D systems, p 2..4, n 32..160, mixed
 // precision): 46, 40 and 35 us with a thread per row -> 27, 26 and 26 us with
@@ -340,11 +348,6 @@ __device__ __forceinline__ void block_columns(double t, const Lanes& L, int Rs, 
     }
 }
 
-// Rows of a grid-stride kernel: a warp per row.
-#define SPMM_ROWS(i, n)                                                         \
-    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < (n);          \
-         i += (gridDim.x * blockDim.x) >> 5)
-
 // ------------------------------------------- kernels, several right-hand sides
 // FP64 residual r = F - K x; x0 = r / d (V-cycle precision); block partials
 // of r^2 and F^2.  due: only the right-hand sides of the mask (a residual
@@ -594,8 +597,11 @@ __global__ void __launch_bounds__(kBlock, 2) k_m_up0(int n, int Rs, int lp, int 
     if (flexible) block_columns<A>(zq, L, Rs, sh, part_zq + (int64_t)blockIdx.x * Rs);
 }
 
-// Threads of the vector kernels: Rs / 2 threads per row (two columns each),
-// kBlock / (Rs / 2) rows of a block at a time.
+// Threads of the vector kernels: Rs / 2 threads per row (two columns each), as many
+// rows of a block at a time as there would be with Rs a multiple of 4: one thread
+// adds a column's terms of those rows one after another (2 right-hand sides, 2-D
+// p = 3 n = 101: 111 us per iteration with 256 rows, 104 with 128).
+__host__ __device__ __forceinline__ int pair_rows(int Rs) { return kBlock / (((Rs + 3) & ~3) >> 1); }
 struct PairLayout {
     int lpr, rpb, rl, c;
     bool in;
@@ -603,7 +609,7 @@ struct PairLayout {
 __device__ __forceinline__ PairLayout pair_layout(int Rs) {
     PairLayout P;
     P.lpr = Rs >> 1;
-    P.rpb = kBlock / P.lpr;
+    P.rpb = pair_rows(Rs);
     P.rl = threadIdx.x / P.lpr;
     P.c = 2 * (threadIdx.x - P.rl * P.lpr);
     P.in = P.rl < P.rpb;
@@ -1066,13 +1072,23 @@ int lanes_per_entry(int Rs) {
     while (p < q) p <<= 1;
     return p;
 }
+// on a level: two where one would do (two FP64 columns) and the rows are short (at
+// most kPairRow entries on average), since 32 groups have more to add up than such
+// a row gives them.  Us per iteration with one / two: 2-D p = 3 n = 101 (49 entries)
+// 104 / 102, 3-D p = 2 n = 12 (90) 57 / 59, p = 3 n = 24 (284) 168 / 221.
+constexpr int kPairRow = 64;
+template <typename A>
+int lanes_per_entry(int Rs, const Level& L) {
+    const int p = lanes_per_entry<A>(Rs);
+    return p == 1 && sizeof(A) == 8 && L.A.nnz <= (int64_t)kPairRow * L.A.n ? 2 : p;
+}
 
 // Rows of a block that share one epilogue: all copies of a column where the
 // level has rows enough to fill the GPU's warps that way, else one.
 template <typename A>
-int rows_together(amg_hierarchy* h, int n, int Rs) {
-    const int t = 32 / (kVec<A> * lanes_per_entry<A>(Rs));
-    return (int64_t)n >= (int64_t)h->num_sms * 16 * t ? t : 1;
+int rows_together(amg_hierarchy* h, const Level& L, int Rs) {
+    const int t = 32 / (kVec<A> * lanes_per_entry<A>(Rs, L));
+    return (int64_t)L.A.n >= (int64_t)h->num_sms * 16 * t ? t : 1;
 }
 
 // blocks of the SpMM kernels: two per SM (the partial sums of a dot product
@@ -1089,7 +1105,7 @@ int coarse_blocks(amg_hierarchy* h) {
 
 // blocks of the vector kernels of R right-hand sides
 int pair_blocks(amg_hierarchy* h, int n, int Rs) {
-    const int rpb = kBlock / (Rs / 2);
+    const int rpb = pair_rows(Rs);
     const int64_t b = ((int64_t)n + rpb - 1) / rpb;
     const int64_t cap = (int64_t)h->num_sms * 2;
     return (int)(b < cap ? b : cap);
@@ -1114,7 +1130,7 @@ template <typename A>
 cudaError_t m_vcycle(amg_hierarchy* h, cudaStream_t s) {
     using Vw = MView<A>;
     MultiWork& w = *h->mw;
-    const int L = h->nlev, Rs = w.Rs, lp = lanes_per_entry<A>(Rs), flex = h->o.flexible;
+    const int L = h->nlev, Rs = w.Rs, flex = h->o.flexible;
     const int* act = w.active;
     if (L == 1) {
         launch_pdl(k_m_coarse<double, A>, coarse_blocks(h), kCoarseWarps * 32, 0, s, h->ndense, Rs,
@@ -1125,7 +1141,7 @@ cudaError_t m_vcycle(amg_hierarchy* h, cudaStream_t s) {
     for (int l = 0; l < L - 1; l++) {
         Level& F = h->lev[l];
         Level& C = h->lev[l + 1];
-        const int n = F.A.n, nb = spmm_blocks(h, n), T = rows_together<A>(h, n, Rs);
+        const int n = F.A.n, nb = spmm_blocks(h, n), T = rows_together<A>(h, F, Rs), lp = lanes_per_entry<A>(Rs, F);
         const bool coarsest = (l + 1 == L - 1);
         A* xc = coarsest ? nullptr : Vw::x(w, l + 1);
         if (l > 0 && n <= nb * kWarpsPerBlock) {  // a warp for every row
@@ -1162,7 +1178,7 @@ cudaError_t m_vcycle(amg_hierarchy* h, cudaStream_t s) {
     }
     for (int l = L - 2; l >= 0; l--) {
         Level& F = h->lev[l];
-        const int n = F.A.n, nb = spmm_blocks(h, n), T = rows_together<A>(h, n, Rs);
+        const int n = F.A.n, nb = spmm_blocks(h, n), T = rows_together<A>(h, F, Rs), lp = lanes_per_entry<A>(Rs, F);
         Vw::vals(F, l, [&](auto vp) {
             using V = vt<decltype(vp)>;
             if (l == 0) {
@@ -1213,8 +1229,8 @@ cudaError_t any_residual(amg_hierarchy* h, double* r, bool x0, bool ff, bool due
     const bool want = x0 && h->nlev > 1;
     const unsigned* gate = due ? w.due : nullptr;
     if (!w.tiles) {
-        const int nb = spmm_blocks(h, n), lp = lanes_per_entry<double>(w.Rs);
-        const int T = rows_together<double>(h, n, w.Rs);
+        const int nb = spmm_blocks(h, n), lp = lanes_per_entry<double>(w.Rs, L0);
+        const int T = rows_together<double>(h, L0, w.Rs);
         double* pff = ff ? mslot(w, M_B) : nullptr;
         const auto mat = mat_of(L0, static_cast<const double*>(L0.A.val));
         if (h->mixed)
@@ -1267,13 +1283,13 @@ cudaError_t any_spmv_pq(amg_hierarchy* h, Parts* P, cudaStream_t s) {
     if (h->mixed)
         with_runs<float>(L0, [&](auto rn) {
             launch_pdl(k_m_spmv_pq<decltype(rn)::value, float, float>, nb, kBlock, 0, s, n, w.Rs,
-                       lanes_per_entry<float>(w.Rs), rows_together<float>(h, n, w.Rs),
+                       lanes_per_entry<float>(w.Rs, L0), rows_together<float>(h, L0, w.Rs),
                        mat_of(L0, static_cast<const float*>(L0.val32)), w.p32, w.p, w.r, w.q, mslot(w, M_A),
                        mslot(w, M_B), flex, w.active);
         });
     else
-        launch_pdl(k_m_spmv_pq<false, double, double>, nb, kBlock, 0, s, n, w.Rs, lanes_per_entry<double>(w.Rs),
-                   rows_together<double>(h, n, w.Rs), mat_of(L0, static_cast<const double*>(L0.A.val)), w.p, w.p,
+        launch_pdl(k_m_spmv_pq<false, double, double>, nb, kBlock, 0, s, n, w.Rs, lanes_per_entry<double>(w.Rs, L0),
+                   rows_together<double>(h, L0, w.Rs), mat_of(L0, static_cast<const double*>(L0.A.val)), w.p, w.p,
                    w.r, w.q, mslot(w, M_A), mslot(w, M_B), flex, w.active);
     *P = spmm_parts(h);
     return cudaGetLastError();
