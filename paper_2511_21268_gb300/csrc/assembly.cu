@@ -414,9 +414,10 @@ __device__ __forceinline__ int tile_at(int slice, int row, int piece) {
 // 32 A rows, and issues 36 digit pairs x 4 MMAs.  Blocks of the same plane
 // points run next to each other (x: the z tiles), so A's digits come from L2.
 // Measured at n = 64, p = 3, M = 256: digits 1.06 ms (bound by cos and sin in
-// FP64), product with the coefficients 2.24 ms (36 digit products, 0.31 P
-// multiply-adds; the coefficients' exp and FP64 products are about half of
-// it), against 1.39 and 16.34 ms in FP64.  The whole assembly 30.0 -> 16.6 ms,
+// FP64), product with the coefficients 2.24 ms (36 digit products, 0.31 T
+// multiply-adds: 0.28 PFLOP/s, 0.14 of the rate a plain 16-bit product reaches;
+// mma.sync's pipe is 45 % busy, the FP64 pipe 31 % with the coefficients' exp and
+// products, 8 warps per SM), against 1.39 and 16.34 ms in FP64.  The whole assembly 30.0 -> 16.6 ms,
 // with the error against a dense FP64 contraction 7.4e-16 before and 7.3e-16
 // after.
 __global__ void __launch_bounds__(256, 1) k_iga_coef_gemm(int64_t P2, int64_t p0, int rows, int Q, int K2, int fix,

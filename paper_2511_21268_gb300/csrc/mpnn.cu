@@ -1301,11 +1301,13 @@ int mpnn_setup_fork(amg_hierarchy* h) {
     return AMG_OK;
 }
 
-// A coarse level that will have a smoother (its matrix and diagonal are
+// A coarse level that is about to be coarsened (its matrix and diagonal are
 // enqueued on the library stream): its features, damping cap and network
 // follow on the second stream, behind the finest level's, while the setup
 // goes on.  At the end of the setup they were a chain of some four hundred
-// small kernels.
+// small kernels.  Should the coarsening stagnate on this level, they were for
+// nothing (at most dense_max rows, and their buffers); to wait until it is known
+// not to took the annulus p = 3 n = 40 from 25.3 to 25.6 ms.
 int mpnn_setup_level(amg_hierarchy* h, int l) {
     if (!h->mp || !h->mp->forked) return AMG_OK;
     MpnnWork& w = *h->mp;

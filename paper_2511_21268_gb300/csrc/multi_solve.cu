@@ -799,7 +799,7 @@ struct Parts {
 // instruction of a warp holds a quarter of an SM's pipe for 64 cycles: 304
 // partials of 16 columns in one block are 2.4 us of adds, on four SMs a quarter.
 // Measured, 16 right-hand sides: alpha 11.1 -> 8.1 us, beta 11.3 -> 8.4, the
-// convergence test 7.6 -> 6.9; a batch of 16: 6.6 -> 4.6, 7.1 -> 5.0, 5.5 -> 4.5.
+// convergence test 7.6 -> 6.9; a batch of 24: 6.1 -> 5.1, 6.4 -> 5.9, 4.9 -> 5.0.
 constexpr int kScalSys = 4;
 
 // Sum of system s's partials on every lane of the warp, in a fixed order.
